@@ -8,14 +8,21 @@
 
 namespace ah {
 
-// Number of z chunks for `tiles` XY tiles of an N-plane lattice when `slots`
-// CTAs are resident at once: the grid runs in waves of `slots` CTAs, each CTA
-// marching its chunk plus `extra` planes of prologue and look-ahead, so
-// minimise ceil(tiles n / slots) (ceil(N / n) + extra) over n with chunks of
-// at least min_chunk planes.
-int choose_chunks(int N, long long tiles, int slots, int min_chunk, int extra = 2);
 // Streaming multiprocessors of the current device (cached per device).
 int device_sm_count();
+// Resident CTAs' time per plane: t[c - 1] for c CTAs on each SM, in any unit (the
+// shape of the curve is what the choice below needs).
+struct PlaneTimes { short t[4]; };
+// Number of z chunks for `tiles` XY tiles of an N-plane lattice, at most `per_sm`
+// (<= 4) CTAs resident on an SM: the grid runs in waves of per_sm CTAs on every SM,
+// each CTA marching its chunk of zc = ceil(N / n) planes plus `extra` planes'
+// worth of prologue, so minimise (zc + extra) (whole waves x t[per_sm] + t[CTAs per
+// SM of the last wave]) over n.  Chunks go down to a single plane: a lattice that
+// cannot fill the GPU is bound by the march of one CTA (64^3, FP32 step: 4 chunks
+// 23.6 us, 32 chunks 10.3 us).  The times matter in
+// between: 3 resident CTAs take less than 3/4 of the time of 4, so at 125^3 seven
+// chunks (39.5 us) beat the nine that fill the wave (41.0 us).
+int choose_chunks(int N, long long tiles, int per_sm, int extra, const PlaneTimes &times);
 
 namespace {
 

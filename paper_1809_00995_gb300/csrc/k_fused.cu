@@ -574,22 +574,6 @@ constexpr VariantInfo kVariants64[] = { { 16, 1, 1, 16, false, "ty16_b1" }, { 8,
 
 }  // namespace
 
-int choose_chunks(int N, long long tiles, int slots, int min_chunk, int extra)
-{
-    const int nmax = std::max(1, std::min(N / std::max(1, min_chunk), 64));
-    int best = 1;
-    long long best_cost = -1;
-    for (int n = 1; n <= nmax; ++n) {
-        const long long waves = (tiles * n + slots - 1) / slots;
-        const long long cost = waves * ((N + n - 1) / n + extra);
-        if (best_cost < 0 || cost < best_cost) {
-            best_cost = cost;
-            best = n;
-        }
-    }
-    return best;
-}
-
 int device_sm_count()
 {
     static int sms[64] = {};
@@ -602,7 +586,31 @@ int device_sm_count()
     return n;
 }
 
+int choose_chunks(int N, long long tiles, int per_sm, int extra, const PlaneTimes &times)
+{
+    const int nmax = std::min(N, 64);
+    const long long sms = device_sm_count(), slots = sms * per_sm;
+    int best = 1;
+    long long best_cost = -1;
+    for (int n = 1; n <= nmax; ++n) {
+        const long long zc = (N + n - 1) / n, ctas = tiles * ((N + zc - 1) / zc);
+        const long long last = ctas % slots;
+        const long long wave = ctas / slots * times.t[per_sm - 1] + (last ? times.t[(last - 1) / sms] : 0);
+        const long long cost = (zc + extra) * wave;
+        if (best_cost < 0 || cost < best_cost) {
+            best_cost = cost;
+            best = n;
+        }
+    }
+    return best;
+}
+
 namespace {
+
+// FP32 step, microseconds x 100 per plane measured at 64^3 to 256^3 (113 with one
+// CTA on an SM, 255 with four)
+constexpr PlaneTimes kStepTimes32 = { { 113, 156, 199, 255 } };
+constexpr PlaneTimes kStepTimes64 = { { 100, 150, 200, 250 } };
 
 template <typename real, int TY, int RX, int MINB>
 cudaError_t launch_shape(const View<real> &v, int N, const KickCoef<real> &c, int min_chunk, bool wave_model,
@@ -625,7 +633,7 @@ cudaError_t launch_shape(const View<real> &v, int N, const KickCoef<real> &c, in
     const int tx = (N + G::TX - 1) / G::TX, ty = (N + TY - 1) / TY;
     int nch;
     if (wave_model) {
-        nch = choose_chunks(N, (long long)tx * ty, device_sm_count() * MINB, min_chunk);
+        nch = choose_chunks(N, (long long)tx * ty, MINB, 1, sizeof(real) == 4 ? kStepTimes32 : kStepTimes64);
     } else {
         // enough z chunks for several waves of CTAs, chunks of at least min_chunk planes
         nch = (int)((16LL * device_sm_count() + (long long)tx * ty - 1) / ((long long)tx * ty));
@@ -728,7 +736,7 @@ void fused_diag_grid(int N, int *tx, int *ty, int *nch, int *zc)
 {
     *tx = (N + 31) / 32;
     *ty = (N + 7) / 8;
-    const int n = choose_chunks(N, (long long)*tx * *ty, 2 * device_sm_count(), 16);   // 2 CTAs / SM
+    const int n = choose_chunks(N, (long long)*tx * *ty, 2, 4, PlaneTimes{ { 255, 255 } });   // 2 CTAs / SM
     *zc = (N + n - 1) / n;
     *nch = (N + *zc - 1) / *zc;
 }

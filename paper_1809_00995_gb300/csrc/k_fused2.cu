@@ -291,6 +291,9 @@ struct Shape2 { int ty, minb; const char *name; };
 constexpr Shape2 kShapes2[] = { { 8, 2, "two_ty8_b2" }, { 8, 3, "two_ty8_b3" }, { 16, 1, "two_ty16_b1" },
                                 { 12, 2, "two_ty12_b2" } };
 
+// two-step pass: nearer to its issue limit with few CTAs than the single step
+constexpr PlaneTimes kStep2Times = { { 150, 180, 210, 270 } };
+
 // WEAK (32-bit site indices only; the caller checks fused2_weak_ok)
 template <int TY, int MINB, bool WEAK = false>
 cudaError_t launch_shape2(const View2<float> &v, int N, const KickCoef<float> &c1, const KickCoef<float> &c2,
@@ -311,7 +314,7 @@ cudaError_t launch_shape2(const View2<float> &v, int N, const KickCoef<float> &c
     }
     const int tx = (N + G::OX - 1) / G::OX, ty = (N + G::OY - 1) / G::OY;
     // each chunk also runs the first step on the planes below and above it
-    int nch = choose_chunks(N, (long long)tx * ty, device_sm_count() * MINB, 16, 4);
+    int nch = choose_chunks(N, (long long)tx * ty, MINB, 4, kStep2Times);
     const int zc = (N + nch - 1) / nch;
     nch = (N + zc - 1) / zc;
     if constexpr (WEAK) {
@@ -395,7 +398,7 @@ void fused2_diag_grid(int N, int *tx, int *ty, int *nch, int *zc)
     using G = Geo2<8>;
     *tx = (N + G::OX - 1) / G::OX;
     *ty = (N + G::OY - 1) / G::OY;
-    const int n = choose_chunks(N, (long long)*tx * *ty, 2 * device_sm_count(), 16, 4);   // 2 CTAs / SM
+    const int n = choose_chunks(N, (long long)*tx * *ty, 2, 4, kStep2Times);
     *zc = (N + n - 1) / n;
     *nch = (N + *zc - 1) / *zc;
 }
