@@ -19,7 +19,8 @@ struct PlaneTimes { short t[4]; };
 // worth of prologue, so minimise (zc + extra) (whole waves x t[per_sm] + t[CTAs per
 // SM of the last wave]) over n.  Chunks go down to a single plane: a lattice that
 // cannot fill the GPU is bound by the march of one CTA (64^3, FP32 step: 4 chunks
-// 23.6 us, 32 chunks 10.3 us).  The times matter in
+// 23.6 us, 32 chunks 10.3 us; 32^3, FP64 step: 2 chunks 236 us, 32
+// chunks 26.7 us).  The times matter in
 // between: 3 resident CTAs take less than 3/4 of the time of 4, so at 125^3 seven
 // chunks (39.5 us) beat the nine that fill the wave (41.0 us).
 int choose_chunks(int N, long long tiles, int per_sm, int extra, const PlaneTimes &times);

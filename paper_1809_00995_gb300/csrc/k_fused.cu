@@ -31,6 +31,7 @@
 #include "diag_common.cuh"
 #include "sincos32.cuh"
 #include "fused_common.cuh"
+#include "step_tile.cuh"
 
 namespace ah {
 namespace {
@@ -485,11 +486,21 @@ __device__ __forceinline__ void fused_tile(const View<real> &v, int N, int zc, c
     diag_flush();
 }
 
+// Shapes that run step_tile instead of fused_tile: FP64, one site per thread.
+// (FP32 issues its link exponentials and plaquette products at 64 times the
+// FP64 rate and waits on memory instead, for which fused_tile keeps one more
+// plane in flight.)
+template <typename real, int TY, int RX>
+constexpr bool kStepTile = sizeof(real) == 8 && TY == 8 && RX == 1;
+
 template <typename real, int TY, int RX, int MINB, typename IT>
 __global__ void __launch_bounds__(256, MINB) k_fused(View<real> v, int N, int zc, KickCoef<real> c)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    fused_tile<real, TY, RX, IT>(v, N, zc, c, blockIdx.x, blockIdx.y, blockIdx.z, smem_raw);
+    if constexpr (kStepTile<real, TY, RX>)
+        step_tile<real, TY, IT>(v, N, zc, c, blockIdx.x, blockIdx.y, blockIdx.z, smem_raw);
+    else
+        fused_tile<real, TY, RX, IT>(v, N, zc, c, blockIdx.x, blockIdx.y, blockIdx.z, smem_raw);
 }
 
 // Diagnostics of the current state through the step's tile walk (tile 32 x 8,
@@ -610,23 +621,25 @@ namespace {
 // FP32 step, microseconds x 100 per plane measured at 64^3 to 256^3 (113 with one
 // CTA on an SM, 255 with four)
 constexpr PlaneTimes kStepTimes32 = { { 113, 156, 199, 255 } };
-constexpr PlaneTimes kStepTimes64 = { { 100, 150, 200, 250 } };
+// FP64 step: bound by the FP64 pipe, which one CTA fills to 0.88
+constexpr PlaneTimes kStepTimes64 = { { 123, 216, 324, 432 } };
 
 template <typename real, int TY, int RX, int MINB>
 cudaError_t launch_shape(const View<real> &v, int N, const KickCoef<real> &c, int min_chunk, bool wave_model,
                          cudaStream_t st)
 {
     using G = Geo<real, TY, RX>;
+    constexpr size_t smem = kStepTile<real, TY, RX> ? TileGeo<real, 8>::smem : G::smem;
     if (RX > 1 && (N & 1)) return cudaErrorInvalidValue;
     const bool idx32 = (long long)N * N * N < (1LL << 31);
     static unsigned long long configured = 0;   // per device, once per instantiation
     const unsigned long long dev_bit = 1ULL << device_slot();
     if (!(configured & dev_bit)) {
         cudaError_t e = cudaFuncSetAttribute(k_fused<real, TY, RX, MINB, int>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::smem);
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_fused<real, TY, RX, MINB, long long>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::smem);
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         configured |= dev_bit;
     }
@@ -641,8 +654,8 @@ cudaError_t launch_shape(const View<real> &v, int N, const KickCoef<real> &c, in
     }
     const int zc = (N + nch - 1) / nch;
     nch = (N + zc - 1) / zc;
-    if (idx32) k_fused<real, TY, RX, MINB, int><<<dim3(tx, ty, nch), G::NT, G::smem, st>>>(v, N, zc, c);
-    else k_fused<real, TY, RX, MINB, long long><<<dim3(tx, ty, nch), G::NT, G::smem, st>>>(v, N, zc, c);
+    if (idx32) k_fused<real, TY, RX, MINB, int><<<dim3(tx, ty, nch), G::NT, smem, st>>>(v, N, zc, c);
+    else k_fused<real, TY, RX, MINB, long long><<<dim3(tx, ty, nch), G::NT, smem, st>>>(v, N, zc, c);
     return cudaGetLastError();
 }
 
@@ -653,7 +666,7 @@ cudaError_t launch_shape(const View<real> &v, int N, const KickCoef<real> &c, in
 template <>
 int fused_default_variant<float>() { return 10; }      // ty8_b4_w
 template <>
-int fused_default_variant<double>() { return 1; }      // ty8_b2
+int fused_default_variant<double>() { return 3; }      // ty8_b2_w
 
 template <>
 int fused_variant_count<float>() { return (int)(sizeof(kVariants32) / sizeof(kVariants32[0])); }

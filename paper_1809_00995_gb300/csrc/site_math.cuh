@@ -1,0 +1,151 @@
+// site_math.cuh -- per-site arithmetic of the leapfrog (Eqs. up_pi, up_E of
+// arXiv:1809.00995) of the FP64 step, with every multiply-add written out
+// (__fma_rn), since the count of FP64 instructions is the time of the step.
+//
+// The plaquette sines come from the link phases themselves,
+//   Xi_ij = (theta_i^x - theta_i^{x+j}) + (theta_j^{x+i} - theta_j^x),
+// instead of from products of four link exponentials: 3 subtractions and an odd
+// polynomial instead of ten multiply-adds on eight values, neighbours exchange
+// one phase instead of a complex exponential, and the halo of a tile needs no
+// sincos of its own except for the one link per site that points into the tile.
+#pragma once
+#include "ah_internal.cuh"
+#include "sincos64.cuh"
+
+namespace ah {
+namespace {
+
+__device__ __forceinline__ double fm(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ double ml(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double ad(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double sb(double a, double b) { return __dsub_rn(a, b); }
+
+template <typename real> struct alignas(2 * sizeof(real)) V2 { real r, i; };
+template <typename real> struct alignas(16) V4 { real a, b, c, d; };
+
+// rounding error of s = fl(a + b) (Knuth)
+__device__ __forceinline__ double two_sum_err(double a, double b, double s)
+{
+    const double bb = sb(s, a);
+    return ad(sb(a, sb(s, bb)), sb(b, bb));
+}
+
+// U phi and conj(U) phi
+template <typename real>
+__device__ __forceinline__ V2<real> fwd(V2<real> u, V2<real> f)
+{
+    return { fm(-u.i, f.i, ml(u.r, f.r)), fm(u.i, f.r, ml(u.r, f.i)) };
+}
+template <typename real>
+__device__ __forceinline__ V2<real> bwd(V2<real> u, V2<real> f)
+{
+    return { fm(u.i, f.i, ml(u.r, f.r)), fm(-u.i, f.r, ml(u.r, f.i)) };
+}
+
+// U = e^{i theta} of NL links of a site (sincos64.cuh; one warp vote picks the
+// range of the polynomials)
+template <int NL>
+__device__ __forceinline__ void link_exps(const double *t, V2<double> *u)
+{
+    int m = abs_hi(t[0]);
+#pragma unroll
+    for (int d = 1; d < NL; ++d) m = max(m, abs_hi(t[d]));
+    const unsigned mm = __reduce_max_sync(__activemask(), (unsigned)m);
+    if (mm <= kHi2m4) {
+#pragma unroll
+        for (int d = 0; d < NL; ++d) sincos_range<0>(t[d], &u[d].i, &u[d].r);
+    } else if (mm <= kHi04) {
+#pragma unroll
+        for (int d = 0; d < NL; ++d) sincos_range<1>(t[d], &u[d].i, &u[d].r);
+    } else if (mm <= kHi078) {
+#pragma unroll
+        for (int d = 0; d < NL; ++d) sincos_range<2>(t[d], &u[d].i, &u[d].r);
+    } else {
+#pragma unroll
+        for (int d = 0; d < NL; ++d) sincos_reduced(t[d], 0.0, &u[d].i, &u[d].r);
+    }
+}
+
+// Sines of NX plaquettes from their phases: Xi = (ti - tij) + (tji - tj), the
+// phases of U_i^x, U_i^{x+j}, U_j^{x+i}, U_j^x.  When every |Xi| of the warp is
+// small the sum is good to an ulp of its largest difference and the odd
+// polynomial applies; beyond, the sum's rounding errors are kept (Knuth's
+// TwoSum) and added after the range reduction, so that a Xi near a multiple of
+// 2 pi (compact phases on the two sides of the cut) loses nothing.
+template <int NX>
+__device__ __forceinline__ void plaq_sines(const double *ti, const double *tij, const double *tj, const double *tji,
+                                           double *p)
+{
+    double x[NX];
+    int m = 0;
+#pragma unroll
+    for (int k = 0; k < NX; ++k) {
+        x[k] = ad(sb(ti[k], tij[k]), sb(tji[k], tj[k]));
+        m = max(m, abs_hi(x[k]));
+    }
+    const unsigned mm = __reduce_max_sync(__activemask(), (unsigned)m);
+    if (mm <= kHi2m4) {
+#pragma unroll
+        for (int k = 0; k < NX; ++k) p[k] = sin_range<0>(x[k]);
+    } else if (mm <= kHi04) {
+#pragma unroll
+        for (int k = 0; k < NX; ++k) p[k] = sin_range<1>(x[k]);
+    } else if (mm <= kHi078) {
+#pragma unroll
+        for (int k = 0; k < NX; ++k) p[k] = sin_range<2>(x[k]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < NX; ++k) {
+            const double a = sb(ti[k], tij[k]), b = sb(tji[k], tj[k]);
+            const double ea = two_sum_err(ti[k], -tij[k], a), eb = two_sum_err(tji[k], -tj[k], b);
+            double c;
+            sincos_reduced(x[k], ad(two_sum_err(a, b, x[k]), ad(ea, eb)), &p[k], &c);
+        }
+    }
+}
+
+// One kick of Pi (Eq. up_pi) and the scalar currents Im[conj(U_d phi^{x+d}) phi^x]
+// of a site: f0 = phi^x, w_d = U_d phi^{x+d}, b_d = conj(U_d^{x-d}) phi^{x-d}.
+template <typename real>
+struct PiKick { real pr, pi, c1, c2, c3; };
+template <typename real>
+__device__ __forceinline__ PiKick<real> pi_kick(const KickCoef<real> &c, V2<real> f0, V2<real> w1, V2<real> w2,
+                                                V2<real> w3, V2<real> b1, V2<real> b2, V2<real> b3, real pr, real pi)
+{
+    const real lr = fm(real(-6), f0.r, ad(ad(ad(w1.r, b1.r), ad(w2.r, b2.r)), ad(w3.r, b3.r)));
+    const real li = fm(real(-6), f0.i, ad(ad(ad(w1.i, b1.i), ad(w2.i, b2.i)), ad(w3.i, b3.i)));
+    const real pot = ml(c.c_pot, sb(fm(f0.r, f0.r, ml(f0.i, f0.i)), c.sigma2));
+    PiKick<real> k;
+    k.pr = fm(c.c_lap, lr, fm(-pot, f0.r, ml(c.c_damp, pr)));
+    k.pi = fm(c.c_lap, li, fm(-pot, f0.i, ml(c.c_damp, pi)));
+    k.c1 = fm(w1.r, f0.i, -ml(w1.i, f0.r));
+    k.c2 = fm(w2.r, f0.i, -ml(w2.i, f0.r));
+    k.c3 = fm(w3.r, f0.i, -ml(w3.i, f0.r));
+    return k;
+}
+
+// Kick of one E component (Eq. up_E) in two parts: everything but the curl,
+// then the curl sum_{j != i} [sin Xi_ij^x - sin Xi_ij^{x-j}], whose terms at the
+// neighbours x - j arrive one barrier later.
+template <typename real>
+__device__ __forceinline__ real e_local(const KickCoef<real> &c, real e, real cur)
+{
+    return fm(c.c_cur, cur, ml(c.c_edamp, e));
+}
+template <typename real>
+__device__ __forceinline__ real e_kick(const KickCoef<real> &c, real local, real curl)
+{
+    return fm(-c.c_curl, curl, local);
+}
+
+// Drift of a link phase, compact if the run asks for it
+template <typename real>
+__device__ __forceinline__ real th_drift(const KickCoef<real> &c, real t, real e)
+{
+    real n = fm(c.dt, e, t);
+    if (c.wrap) n = wrap_phase(n);
+    return n;
+}
+
+}  // namespace
+}  // namespace ah
