@@ -437,9 +437,6 @@ ah_status do_diag(ah_sim *h, Box b, ah_obs *out)
     const View<real> v = make_view(F, h->cur, false);
     const bool exact = (h->cfg.flags & AH_FLAG_EXACT_DIAG) != 0;
     const bool whole = b.x0 == 0 && b.y0 == 0 && b.z0 == 0 && b.nx == h->N && b.ny == h->N && b.nz == h->N;
-    if (whole && !exact && fused_diag_ctas(h->N) > h->nparts)
-        return fail(AH_ERR_CUDA, "diagnostics scratch too small: the N=%d pass needs %d partials, %d allocated",
-                    h->N, fused_diag_ctas(h->N), h->nparts);
     if (whole && !exact)
         AH_CUDA(launch_diag_whole<real>(v, h->N, dc, h->partials, h->nparts, h->result, h->list, h->diag_blocks,
                                         h->stream));
@@ -569,9 +566,6 @@ ah_status diag_start(ah_sim *h)
         AH_CUDA(launch_diag<real>(v, N, Box{ 0, 0, 0, N, N, N }, dc, h->partials, h->diag_blocks, h->result, h->list,
                                   true, h->aux));
     } else {
-        if (fused_diag_ctas(N) > h->nparts)
-            return fail(AH_ERR_CUDA, "diagnostics scratch too small: the N=%d pass needs %d partials, %d allocated", N,
-                        fused_diag_ctas(N), h->nparts);
         AH_CUDA(launch_diag_whole<real>(v, N, dc, h->partials, h->nparts, h->result, h->list, h->diag_blocks, h->aux));
         // a list overflow is settled on the device: the snapshot may change
         // before the host could look at the count
@@ -647,7 +641,7 @@ ah_status ah_create_ex(const ah_config *cfg, ah_sim **out)
     const size_t esz = cfg->precision == AH_FP32 ? sizeof(float) : sizeof(double);
     h->dbytes = (h->two_step ? 20 : 15) * padded((size_t)h->nsites) * esz;
     h->diag_blocks = diag_grid_blocks(h->num_sms);
-    const int nparts = std::max({ h->diag_blocks, fused_diag_ctas(h->N), h->two_step ? fused2_diag_ctas(h->N) : 0 });
+    const int nparts = std::max({ h->diag_blocks, fused_diag_max_ctas(), h->two_step ? fused2_diag_ctas(h->N) : 0 });
     h->nparts = nparts;
     // expected near-cut plaquettes: about 5e-5 of the 3 N^3 plaquettes in FP32
     h->list.capacity = std::max<long long>(1LL << 20, h->nsites * 3 / 2000);

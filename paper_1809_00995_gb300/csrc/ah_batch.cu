@@ -202,13 +202,7 @@ struct Engine {
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev);
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
         diag_blocks = diag_grid_blocks(num_sms);
-        // partials of the whole-lattice pass: the most CTAs that any accepted
-        // lattice side needs (the z-chunk count of the pass depends on N, so the
-        // largest N does not give the largest grid: 1024^3 takes more CTAs
-        // than 1290^3)
-        int max_ctas = 0;
-        for (int n = 4; n <= kMaxBatchN; ++n) max_ctas = std::max(max_ctas, fused_diag_ctas(n));
-        nparts = std::max(diag_blocks, max_ctas);
+        nparts = std::max(diag_blocks, fused_diag_max_ctas());
         list.capacity = 1 << 20;
         if (e == cudaSuccess) e = cudaMalloc(&d_partials, sizeof(DiagPartial) * (nparts + 1));
         if (e == cudaSuccess) e = cudaMalloc(&list.count, sizeof(unsigned long long) * (1 + list.capacity));
@@ -469,12 +463,6 @@ struct Engine {
         const View<float> v = lat_view(L);
         const Box b{ 0, 0, 0, L.N, L.N, L.N };
         const DiagCoef dc = host_diag_coef(L.cfg, L.step);
-        if (fused_diag_ctas(L.N) > nparts) {
-            char msg[160];
-            snprintf(msg, sizeof msg, "diagnostics scratch too small: the N=%d pass needs %d partials, %d allocated",
-                     L.N, fused_diag_ctas(L.N), nparts);
-            return host_fail(AH_ERR_CUDA, msg);
-        }
         cudaError_t e = launch_diag_whole<float>(v, L.N, dc, d_partials, nparts, d_result, list, diag_blocks, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(h_result, d_result, sizeof(DiagPartial), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess)

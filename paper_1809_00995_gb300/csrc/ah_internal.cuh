@@ -178,24 +178,22 @@ template <typename real>
 cudaError_t launch_wind_recount_on_overflow(const View<real> &v, int N, DiagList list, DiagPartial *result,
                                             int nblocks, cudaStream_t st);
 
-// Whole-lattice diagnostics through the fused step's tile walk (tile 32 x 8,
-// nothing written back): one DiagPartial per CTA of the grid that
-// fused_diag_grid gives (fused_diag_ctas of them), near-cut plaquettes
-// appended to the list.
+// Whole-lattice diagnostics on a z-marching tile walk (diag_tile.cuh): one
+// DiagPartial per persistent CTA (at most fused_diag_max_ctas of them,
+// whatever N), near-cut
+// plaquettes appended to the list.
 struct DiagArgs {
     DiagCoef dc;
     DiagPartial *partials;
     DiagList list;
 };
-void fused_diag_grid(int N, int *tx, int *ty, int *nch, int *zc);
-int fused_diag_ctas(int N);
+int fused_diag_max_ctas();
 template <typename real>
 cudaError_t launch_fused_diag(const View<real> &v, int N, const DiagArgs &da, cudaStream_t st);
 // The whole fast diagnostic: clear the list, launch_fused_diag, sum the
 // partials in a fixed order into *result, FP64 windings of the listed
 // plaquettes (fix_blocks x 128 threads).  partials holds `capacity` entries;
-// cudaErrorInvalidValue (nothing launched) if the N^3 pass needs more
-// (fused_diag_ctas(N), which is not monotonic in N).
+// cudaErrorInvalidValue (nothing launched) if the pass needs more.
 template <typename real>
 cudaError_t launch_diag_whole(const View<real> &v, int N, const DiagCoef &c, DiagPartial *partials,
                               int capacity, DiagPartial *result, DiagList list, int fix_blocks, cudaStream_t st);

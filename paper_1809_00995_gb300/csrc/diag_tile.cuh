@@ -1,0 +1,421 @@
+// diag_tile.cuh -- the whole-lattice diagnostics of one state (Sec. 2 of
+// arXiv:1809.00995) on a tile, marched in z: energy sums, Gauss residual and
+// plaquette windings, nothing written back.
+//
+// A CTA of 256 threads takes 32 x 8 columns of sites, a chunk of z planes at a
+// time, and keeps its sums in registers over all the columns it takes; each site
+// is one thread's.  Per plane and site: the three forward products U_d phi^{x+d}
+// (the gradient energy), the three plaquette phases from the link phases
+// (1 - cos Xi by its own series, without cancellation or division), and the
+// Gauss residual (double-float for FP32 states).
+//
+// Windings without arctangents per edge.  With alpha = arg phi of each site, the
+// bracket of Eq. 9 on link e from a to b is [alpha_b - alpha_a + theta_e] =
+// alpha_b - alpha_a + theta_e - 2 pi n_e, n_e the nearest integer of that over
+// 2 pi; around a plaquette the alphas cancel, so
+//   W = (sum of the four brackets - [Xi]) / 2 pi = N - (n_1 + n_2 - n_3 - n_4),
+// N the nearest integer of Xi / 2 pi: one arctangent per site and small integers.
+// alpha is good to 1e-6 in FP32; where a bracket or [Xi] comes within 2^-15 of
+// +-pi (kCutMargin), or phi is too small or too large for alpha, the plaquette goes
+// to the list that the FP64 path decides, so the counts are those of the FP64
+// formula on the same state.  A site needs n_2, n_3 of x + 1 and n_1, n_3 of x + y
+// (one packed word each) and its own n_1, n_2 of the next plane, so the windings
+// of plane z - 1 are summed while plane z is worked on, and a plane costs one
+// barrier (two copies of the shared arrays).
+#pragma once
+#include "diag_common.cuh"
+#include "fused_common.cuh"
+#include "sincos32.cuh"
+#include "sincos64.cuh"
+
+namespace ah {
+namespace {
+
+constexpr float kCutMargin = 1.0f / 32768.0f;
+constexpr float kPi32 = 3.14159265f, kTwoPi32 = 6.28318531f, kInvTwoPi32 = 0.159154943f;
+
+// atan(a) / a on [0, 1] as a polynomial in a^2 (interpolated at the Chebyshev
+// nodes; largest error of atan 4.3e-7)
+__device__ __forceinline__ float atan_unit(float a)
+{
+    const float u = a * a;
+    float p = fmaf(u, 7.648353930562735e-03f, -3.636043146252632e-02f);
+    p = fmaf(u, p, 8.312645554542542e-02f);
+    p = fmaf(u, p, -1.344786435365677e-01f);
+    p = fmaf(u, p, 1.9872039556503296e-01f);
+    p = fmaf(u, p, -3.332567811012268e-01f);
+    p = fmaf(u, p, 9.999992251396179e-01f);
+    return a * p;
+}
+// arg phi to about 1e-6, or NaN where phi is too small, too large or not a number
+__device__ __forceinline__ float site_phase(float r, float i)
+{
+    const float x = fabsf(r), y = fabsf(i), hi = fmaxf(x, y), lo = fminf(x, y);
+    float a = atan_unit(__fdividef(lo, hi));
+    a = y > x ? 0.5f * kPi32 - a : a;
+    a = r < 0.f ? kPi32 - a : a;
+    a = i < 0.f ? -a : a;
+    return hi > 1e-30f && hi < 1e30f && lo >= 0.f ? a : __int_as_float(0x7fc00000);
+}
+
+// n of one link and whether its bracket is too near the cut; k: whole turns
+// already taken from theta
+__device__ __forceinline__ int turns(float a, bool *cut)
+{
+    const float k = rintf(a * kInvTwoPi32);
+    *cut = !(fabsf(fmaf(-k, kTwoPi32, a)) <= kPi32 - kCutMargin);
+    return (int)k;
+}
+// n_1, n_2, n_3 as 9-bit fields and their cut flags; links with more than 255
+// turns count as near the cut
+struct LinkTurns { int n; bool cut; };
+__device__ __forceinline__ LinkTurns link_turns(float a, float b, float theta)
+{
+    LinkTurns t;
+    if (fabsf(theta) <= 8.f) {
+        t.n = turns(b - a + theta, &t.cut);
+    } else {
+        // whole turns out of a large phase first
+        const float k = rintf(theta * kInvTwoPi32);
+        const float r = fmaf(k, 1.74845553e-7f, fmaf(-k, 6.28318548f, theta));
+        t.n = turns(b - a + r, &t.cut);
+        t.cut = t.cut || !(fabsf(k) < 250.f);
+        t.n += t.cut ? 0 : (int)k;
+    }
+    if (t.cut) t.n = 0;
+    return t;
+}
+__device__ __forceinline__ unsigned pack_turns(LinkTurns a, LinkTurns b, LinkTurns c)
+{
+    return (unsigned)((a.n & 511) | (b.n & 511) << 9 | (c.n & 511) << 18) | (unsigned)a.cut << 27 |
+           (unsigned)b.cut << 28 | (unsigned)c.cut << 29;
+}
+__device__ __forceinline__ int turn_of(unsigned w, int d) { return (int)(w << (23 - 9 * d)) >> 23; }
+__device__ __forceinline__ bool cut_of(unsigned w, int d) { return (w >> (27 + d)) & 1u; }
+
+// 1 - cos Xi summed over the three plaquettes of a site, the whole turns N of each
+// and the plaquettes whose [Xi] is too near the cut, from the four phases of each
+// (as in Eq. 3: ti, tj at x, tij = theta_i^{x+j}, tji = theta_j^{x+i})
+struct XiTerms { int n[3]; int cut; };
+__device__ __forceinline__ float xi_terms(const float *ti, const float *tij, const float *tj, const float *tji,
+                                          XiTerms *o)
+{
+    float x[3], m = 0.f, sum = 0.f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        x[k] = (ti[k] - tij[k]) + (tji[k] - tj[k]);
+        m = fmaxf(m, fabsf(x[k]));
+        o->n[k] = 0;
+    }
+    o->cut = 0;
+    if (__all_sync(__activemask(), m <= 0.78f)) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            // through x^8 / 8!: the next term is below 1e-8 of the sum
+            const float u = x[k] * x[k];
+            float p = fmaf(u, -2.480158764e-05f, 1.388888923e-03f);
+            p = fmaf(u, p, -4.166666791e-02f);
+            sum = fmaf(u, fmaf(u, p, 0.5f), sum);
+        }
+        return sum;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const DF d1 = two_sum(ti[k], -tij[k]), d2 = two_sum(tji[k], -tj[k]), d3 = two_sum(d1.h, d2.h);
+        const float lo = d3.l + (d1.l + d2.l);
+        const float kf = rintf(d3.h * kInvTwoPi32);
+        // [Xi] = Xi - 2 pi k with 2 pi in two parts
+        const float r = fmaf(kf, 1.74845553e-7f, fmaf(-kf, 6.28318548f, d3.h)) + lo;
+        const bool cut = !(fabsf(r) <= kPi32 - kCutMargin) || !(fabsf(kf) < 1e6f);
+        o->cut |= cut << k;
+        o->n[k] = cut ? 0 : (int)kf;
+        float s, c;
+        sincos_link(0.5f * r, &s, &c);
+        sum = fmaf(2.f * s, s, sum);
+    }
+    return sum;
+}
+__device__ __forceinline__ double xi_terms(const double *ti, const double *tij, const double *tj, const double *tji,
+                                           XiTerms *o)
+{
+    double x[3], sum = 0.0;
+    int m = 0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        x[k] = (ti[k] - tij[k]) + (tji[k] - tj[k]);
+        m = max(m, abs_hi(x[k]));
+        o->n[k] = 0;
+    }
+    o->cut = 0;
+    const unsigned mm = __reduce_max_sync(__activemask(), (unsigned)m);
+    if (mm <= kHi04) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) sum += mm <= kHi2m4 ? vers_range<0>(x[k]) : vers_range<1>(x[k]);
+        return sum;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float xf = (float)x[k], kf = rintf(xf * kInvTwoPi32);
+        const float r = fmaf(kf, 1.74845553e-7f, fmaf(-kf, 6.28318548f, xf));
+        const bool cut = !(fabsf(r) <= kPi32 - kCutMargin - 1e-6f * fabsf(kf)) || !(fabsf(kf) < 1e2f);
+        o->cut |= cut << k;
+        o->n[k] = cut ? 0 : (int)kf;
+        double s, c;
+        sincos_reduced(0.5 * x[k], 0.0, &s, &c);
+        sum += 2.0 * s * s;
+    }
+    return sum;
+}
+
+__device__ __forceinline__ void diag_links(const float t[3], float s[3], float c[3]) { sincos_link3(t, s, c); }
+__device__ __forceinline__ void diag_links(const double t[3], double s[3], double c[3])
+{
+    const unsigned m = __reduce_max_sync(__activemask(), (unsigned)abs_hi3(t));
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        if (m <= kHi04) sincos_range<1>(t[d], &s[d], &c[d]);
+        else if (m <= kHi078) sincos_range<2>(t[d], &s[d], &c[d]);
+        else sincos_reduced(t[d], 0.0, &s[d], &c[d]);
+    }
+}
+
+template <typename real> struct alignas(16) D4 { real a, b, c, d; };
+template <typename real> struct alignas(2 * sizeof(real)) D2 { real a, b; };
+
+struct DiagGeo {
+    static constexpr int TX = 32, TY = 8, NT = 256, EX = TX + 2, NE = EX * (TY + 2);
+    // two copies of: { phi.re, phi.im, theta_3, theta_2 }, { E_1, E_2 }, theta_1,
+    // alpha, packed turns
+    template <typename real> static constexpr int bytes = NE * (7 * (int)sizeof(real) + 8);
+    template <typename real> static constexpr size_t smem = 2 * (size_t)((bytes<real> + 15) / 16 * 16);
+};
+
+template <typename real, typename IT>
+struct DiagTile {
+    using G = DiagGeo;
+    static constexpr int EX = G::EX, NE = G::NE;
+    // sums 3..13 of ah_obs (compensated for FP32), Gauss sums and maxima, windings
+    Acc<real> s[11];
+    double dg2 = 0.0, dgs2 = 0.0, dgmax = 0.0;
+    Acc<float> fg2, fgs2;
+    DF fgmax{ 0.f, 0.f };
+    real tmax = real(0);
+    int ic[kNumInt] = { 0, 0, 0, 0, 0, 0, 0, 0 };
+
+    // one column of tiles: planes [z0, z1) of the 32 x 8 sites at (x0, y0)
+    __device__ __forceinline__ void column(const View<real> &v, int N, const DiagArgs &da, DF g_div, DF g_phi, int x0,
+                                           int y0, int z0, int z1, unsigned char *smem)
+    {
+        const int lx = threadIdx.x & 31, wy = threadIdx.x >> 5;
+        const IT NN = (IT)N * (IT)N;
+        const bool own = x0 + lx < N && y0 + wy < N;
+        const int roff = wrapm(x0 + lx, N) + N * wrapm(y0 + wy, N);
+        const int e = (wy + 1) * EX + lx + 1;
+        // the ring: phi, theta of the row above (warp 7) and of the column to the
+        // right with the corner between them (warp 3); E_2 of the row below (warp
+        // 0), E_1 of the column to the left (warp 4)
+        const bool above = wy == 7, right = wy == 3 && lx <= 8, fwd = above || right;
+        const bool back = wy == 0 || (wy == 4 && lx < 8);
+        const int rx = wy == 3 ? 32 : wy == 4 ? -1 : lx, ry = wy == 7 ? 8 : wy == 0 ? -1 : lx;
+        const bool ring = fwd || back;
+        const int hoff = wrapm(x0 + rx, N) + N * wrapm(y0 + ry, N);
+        const int he = ring ? (ry + 1) * EX + rx + 1 : 0;
+        const int half = (G::bytes<real> + 15) / 16 * 16;
+        auto at4 = [&](int b) { return reinterpret_cast<D4<real> *>(smem + b * half); };
+        auto at2 = [&](int b) { return reinterpret_cast<D2<real> *>(smem + b * half + NE * 4 * sizeof(real)); };
+        auto at1 = [&](int b) { return reinterpret_cast<real *>(smem + b * half + NE * 6 * sizeof(real)); };
+        auto atf = [&](int b) { return reinterpret_cast<float *>(smem + b * half + NE * 7 * sizeof(real)); };
+        auto atw = [&](int b) { return reinterpret_cast<unsigned *>(smem + b * half + NE * (7 * sizeof(real) + 4)); };
+        auto wrapz = [&](int z) { return (IT)(z < 0 ? z + N : (z >= N ? z - N : z)) * NN; };
+
+        // fields of the next plane, momenta of the current one
+        real nf[2], nt[3], rf[2], rt[3], pr, pim, e1, e2, e3, re = real(0);
+        auto load_fields = [&](int z) {
+            const IT a = wrapz(z) + (IT)roff;
+            nf[0] = v.phr[a]; nf[1] = v.phi[a];
+            nt[0] = v.th1[a]; nt[1] = v.th2[a]; nt[2] = v.th3[a];
+            if (fwd) {
+                const IT b = wrapz(z) + (IT)hoff;
+                rf[0] = v.phr[b]; rf[1] = v.phi[b];
+                rt[0] = v.th1[b]; rt[1] = v.th2[b]; rt[2] = v.th3[b];
+            }
+        };
+        auto load_momenta = [&](int z) {
+            const IT a = wrapz(z) + (IT)roff;
+            pr = v.pir[a]; pim = v.pii[a];
+            e1 = v.e1[a]; e2 = v.e2[a]; e3 = v.e3[a];
+            if (back) re = wy == 0 ? v.e2[wrapz(z) + (IT)hoff] : v.e1[wrapz(z) + (IT)hoff];
+        };
+        real f0[2], t0[3], g0[3];
+        float a0, ra;
+        real e3m = v.e3[wrapz(z0 - 1) + (IT)roff];
+        load_fields(z0);
+        load_momenta(z0);
+        a0 = site_phase((float)nf[0], (float)nf[1]);
+        ra = fwd ? site_phase((float)rf[0], (float)rf[1]) : 0.f;
+        unsigned wm = 0;                         // own turns of plane z - 1
+        XiTerms xm{ { 0, 0, 0 }, 0 };
+        for (int z = z0; z <= z1; ++z) {
+            const int b = z & 1;
+            f0[0] = nf[0]; f0[1] = nf[1];
+            t0[0] = nt[0]; t0[1] = nt[1]; t0[2] = nt[2];
+            g0[0] = rt[0]; g0[1] = rt[1]; g0[2] = rt[2];
+            at4(b)[e] = { f0[0], f0[1], t0[2], t0[1] };
+            at2(b)[e] = { e1, e2 };
+            at1(b)[e] = t0[0];
+            atf(b)[e] = a0;
+            if (fwd) {
+                at4(b)[he] = { rf[0], rf[1], rt[2], rt[1] };
+                at1(b)[he] = rt[0];
+                atf(b)[he] = ra;
+            }
+            if (back) {
+                if (wy == 0) at2(b)[he].b = re;
+                else at2(b)[he].a = re;
+            }
+            const real mpr = pr, mpi = pim, m1 = e1, m2 = e2, m3 = e3;
+            if (z < z1) load_fields(z + 1);
+            __syncthreads();
+
+            const D4<real> qx = at4(b)[e + 1], qy = at4(b)[e + EX];
+            const real t1y = at1(b)[e + EX];
+            const float ax = atf(b)[e + 1], ay = atf(b)[e + EX];
+            const real e1x = at2(b)[e - 1].a, e2y = at2(b)[e - EX].b;
+            if (z + 1 < z1) load_momenta(z + 1);
+            const float an = z < z1 ? site_phase((float)nf[0], (float)nf[1]) : 0.f;
+            const LinkTurns n1 = link_turns(a0, ax, (float)t0[0]), n2 = link_turns(a0, ay, (float)t0[1]);
+            const LinkTurns n3 = link_turns(a0, an, (float)t0[2]);
+            const unsigned w = pack_turns(n1, n2, n3);
+            atw(b)[e] = w;
+            if (fwd) {
+                // the row above: n_1, n_3; the column to the right: n_2, n_3
+                const float rn = z < z1 ? site_phase((float)rf[0], (float)rf[1]) : 0.f;
+                const float aj = above ? atf(b)[he + 1] : (lx < 8 ? atf(b)[he + EX] : 0.f);
+                const LinkTurns k = link_turns(ra, aj, (float)(above ? g0[0] : g0[1]));
+                atw(b)[he] = pack_turns(k, k, link_turns(ra, rn, (float)g0[2]));
+                ra = rn;
+            }
+            // windings of plane z - 1 (Eq. 9): its neighbours' turns are in the other copy
+            if (z > z0 && own) {
+                const unsigned wx = atw(1 - b)[e + 1], wyv = atw(1 - b)[e + EX];
+                const int o1 = turn_of(wm, 0), o2 = turn_of(wm, 1), o3 = turn_of(wm, 2);
+                const int q12 = xm.n[0] - (o1 + turn_of(wx, 1) - turn_of(wyv, 0) - o2);
+                const int q13 = xm.n[1] - (o1 + turn_of(wx, 2) - n1.n - o3);
+                const int q23 = xm.n[2] - (o2 + turn_of(wyv, 2) - n2.n - o3);
+                const unsigned c1 = wm >> 27, cx = wx >> 27, cy = wyv >> 27;     // bits 0, 1, 2: links 1, 2, 3
+                const bool b12 = (c1 & 3) | (cx & 2) | (cy & 1) | (xm.cut & 1);
+                const bool b13 = (c1 & 5) | (cx & 4) | (unsigned)n1.cut | (xm.cut & 2);
+                const bool b23 = (c1 & 6) | (cy & 4) | (unsigned)n2.cut | (xm.cut & 4);
+                const int q[3] = { b12 ? 0 : q12, b13 ? 0 : q13, b23 ? 0 : q23 };
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    ic[k] += abs(q[k]);
+                    ic[3 + k] += q[k];
+                    ic[6] += q[k] != 0;
+                }
+                if (b12 | b13 | b23) {
+                    const bool bad[3] = { b12, b13, b23 };
+                    const unsigned long long site =
+                        (unsigned long long)((long long)(z - 1) * N * (long long)N + (long long)roff);
+#pragma unroll
+                    for (int k = 0; k < 3; ++k)
+                        if (bad[k]) {
+                            const unsigned long long i = atomicAdd(da.list.count, 1ULL);
+                            if (i < (unsigned long long)da.list.capacity) da.list.items[i] = site * 4ULL + k;
+                        }
+                }
+            }
+            if (z == z1) break;
+            // energies and the Gauss residual of plane z
+            XiTerms xt;
+            {
+                const real ti[3] = { t0[0], t0[0], t0[1] }, tij[3] = { t1y, nt[0], nt[1] };
+                const real tj[3] = { t0[1], t0[2], t0[2] }, tji[3] = { qx.d, qx.c, qy.c };
+                const real bsum = xi_terms(ti, tij, tj, tji, &xt);
+                real sn[3], co[3];
+                diag_links(t0, sn, co);
+                if (own) site(da, g_div, g_phi, f0, t0, sn, co, qx, qy, nf, bsum, mpr, mpi, m1, m2, m3, e1x, e2y, e3m);
+            }
+            xm = xt;
+            wm = w;
+            e3m = m3;
+            a0 = an;
+        }
+        __syncthreads();                         // the next column reuses the arrays
+    }
+
+    __device__ __forceinline__ void site(const DiagArgs &da, DF g_div, DF g_phi, const real f0[2], const real t0[3],
+                                         const real sn[3], const real co[3], const D4<real> &qx, const D4<real> &qy,
+                                         const real nf[2], real bsum, real pr, real pim, real e1, real e2, real e3,
+                                         real e1b, real e2b, real e3b)
+    {
+        const DiagCoef &dc = da.dc;
+        const real fr[3] = { qx.a, qy.a, nf[0] }, fi[3] = { qx.b, qy.b, nf[1] };
+        real g = real(0);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const real wr = co[d] * fr[d] - sn[d] * fi[d], wi = co[d] * fi[d] + sn[d] * fr[d];
+            const real a = wr - f0[0], b = wi - f0[1];
+            g += a * a + b * b;
+        }
+        const real K = pr * pr + pim * pim;
+        const real G2 = g * (real)dc.inv_dx2;
+        const real m2 = f0[0] * f0[0] + f0[1] * f0[1] - (real)dc.sigma2;
+        const real V = (real)dc.v_coef * m2 * m2;
+        const real Eel = (real)dc.eel_coef * (e1 * e1 + e2 * e2 + e3 * e3);
+        const real B = (real)dc.b_coef * bsum;
+        const real L = K - G2 - V + Eel - B;
+        const real rho = K + G2 + V + Eel + B;
+        const real pp = K - G2 * real(1.0 / 3.0) - V + (Eel + B) * real(1.0 / 3.0);
+        s[0].add(K); s[1].add(G2); s[2].add(V); s[3].add(Eel); s[4].add(B);
+        s[5].add(K * V); s[6].add(G2 * V); s[7].add(K * L); s[8].add(G2 * L); s[9].add(pp * L); s[10].add(rho * L);
+        tmax = fmax(tmax, fmax(fabs(t0[0]), fmax(fabs(t0[1]), fabs(t0[2]))));
+        ic[7] += !(isfinite(L) && isfinite(rho) && isfinite(pp));
+        if constexpr (sizeof(real) == 8) {
+            const double div = (e1 - e1b) + (e2 - e2b) + (e3 - e3b);
+            const double g1 = dc.g_div * div;
+            const double g2 = dc.g_phi * (f0[0] * pim - f0[1] * pr);
+            const double Gs = g1 + g2, gs = fabs(g1) + fabs(g2);
+            dg2 += Gs * Gs;
+            dgs2 += gs * gs;
+            dgmax = fmax(dgmax, fabs(Gs));
+        } else {
+            const DF div = df_add(df_add(two_sum(e1, -e1b), two_sum(e2, -e2b)), two_sum(e3, -e3b));
+            const DF a = two_prod(f0[0], pim), b = two_prod(f0[1], pr);
+            const DF g1 = df_mul(g_div, div), g2 = df_mul(g_phi, df_add(a, { -b.h, -b.l }));
+            DF Gs = df_add(g1, g2);
+            if (Gs.h < 0.f) Gs = { -Gs.h, -Gs.l };
+            const float gs = fabsf(g1.h) + fabsf(g2.h);
+            const float sg = Gs.h * 0x1p30f, ss = gs * 0x1p30f;
+            fg2.add(sg * sg);
+            fgs2.add(ss * ss);
+            if (Gs.h > fgmax.h || (Gs.h == fgmax.h && Gs.l > fgmax.l)) fgmax = Gs;
+        }
+    }
+
+    __device__ __forceinline__ void flush(DiagPartial *out)
+    {
+        double accd[kNumSums];
+#pragma unroll
+        for (int k = 3; k < 14; ++k) accd[k] = s[k - 3].value();
+        // the sums of L, rho and p are linear in those of K, G2, V, E_el, B
+        accd[0] = accd[3] - accd[4] - accd[5] + accd[6] - accd[7];
+        accd[1] = accd[3] + accd[4] + accd[5] + accd[6] + accd[7];
+        accd[2] = accd[3] - accd[4] * (1.0 / 3.0) - accd[5] + (accd[6] + accd[7]) * (1.0 / 3.0);
+        if constexpr (sizeof(real) == 4) {
+            dg2 = fg2.value() * 0x1p-60;
+            dgs2 = fgs2.value() * 0x1p-60;
+            dgmax = (double)fgmax.h + (double)fgmax.l;
+        }
+        accd[14] = dg2;
+        accd[15] = dgs2;
+        double mx[kNumMax] = { dgmax, (double)tmax };
+        long long il[kNumInt];
+#pragma unroll
+        for (int k = 0; k < kNumInt; ++k) il[k] = ic[k];
+        block_reduce<256>(accd, mx, il, out);
+    }
+};
+
+}  // namespace
+}  // namespace ah

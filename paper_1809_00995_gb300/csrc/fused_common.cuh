@@ -63,10 +63,6 @@ struct Geo {
     static constexpr int PX = TX + 1, PY = TY + 1, NP = PX * PY;
     static constexpr int NPHALO = PX + TY;
     static constexpr size_t smem = sizeof(cpx<real>) * (2 * 3 * NE + 2 * NE) + sizeof(real) * 3 * NP;
-    // MODE_DIAG: the three scaled edge products of each site of plane z
-    // (tile, right column, top row) after the step's arrays
-    static constexpr size_t diag_off = (smem + 15) / 16 * 16;
-    static constexpr size_t smem_diag = diag_off + sizeof(cpx<real>) * 3 * NE;
     static_assert(TY % 8 == 0 && NHALO <= NT && NPHALO <= NT && TX + TY <= NT, "tile shape");
 };
 

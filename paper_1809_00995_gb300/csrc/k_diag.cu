@@ -38,6 +38,7 @@
 
 #include "ah_internal.cuh"
 #include "diag_common.cuh"
+#include "diag_tile.cuh"
 #include "sincos32.cuh"
 
 namespace ah {
@@ -340,25 +341,6 @@ __global__ void __launch_bounds__(NT) k_diag_exact(View<real> v, int N, Box b, D
     block_reduce<NT>(acc, mx, ic, &partials[blockIdx.x]);
 }
 
-// Sum the partials in index order (one block; thread k owns one output).
-__global__ void k_diag_finish(const DiagPartial *partials, int n, DiagPartial *result)
-{
-    const int k = threadIdx.x;
-    if (k < kNumSums) {
-        double s = 0.0;
-        for (int b = 0; b < n; ++b) s += partials[b].sums[k];
-        result->sums[k] = s;
-    } else if (k < kNumSums + kNumMax) {
-        double m = 0.0;
-        for (int b = 0; b < n; ++b) m = fmax(m, partials[b].maxv[k - kNumSums]);
-        result->maxv[k - kNumSums] = m;
-    } else if (k < kNumSums + kNumMax + kNumInt) {
-        long long s = 0;
-        for (int b = 0; b < n; ++b) s += partials[b].ints[k - kNumSums - kNumMax];
-        result->ints[k - kNumSums - kNumMax] = s;
-    }
-}
-
 // Sum many partials in a fixed order: lane k of warp c reduces word k of
 // partials [c n/32, (c+1) n/32), then thread k adds the 32 chunk results.
 __global__ void __launch_bounds__(1024) k_diag_sum(const DiagPartial *partials, int n, DiagPartial *result)
@@ -402,12 +384,76 @@ __global__ void __launch_bounds__(1024) k_diag_sum(const DiagPartial *partials, 
 
 int diag_grid_blocks(int num_sms) { return num_sms * 4; }
 
+// ------------------------------------------------------------------ whole lattice
+namespace {
+// Persistent CTAs over the work items (tile column, chunk of z planes), each
+// taking every gridDim.x-th one; one partial per CTA.
+template <typename real, typename IT, int MINB>
+__global__ void __launch_bounds__(256, MINB)
+    k_diag_whole(View<real> v, int N, int tx, int ty, int items, int zc, DF g_div, DF g_phi, DiagArgs da)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    DiagTile<real, IT> t;
+    for (int it = blockIdx.x; it < items; it += gridDim.x) {
+        const int bx = it % tx, by = (it / tx) % ty, z0 = it / (tx * ty) * zc;
+        t.column(v, N, da, g_div, g_phi, 32 * bx, 8 * by, z0, min(z0 + zc, N), smem_raw);
+    }
+    t.flush(&da.partials[blockIdx.x]);
+}
+
+// CTAs per SM that the registers allow
+template <typename real> constexpr int kDiagCtas = sizeof(real) == 4 ? 2 : 1;
+
+struct DiagGrid { int tx, ty, zc, items, ctas; };
+template <typename real>
+DiagGrid diag_whole_grid(int N)
+{
+    DiagGrid g;
+    g.tx = (N + 31) / 32;
+    g.ty = (N + 7) / 8;
+    const int n = choose_chunks(N, (long long)g.tx * g.ty, kDiagCtas<real>, 1, PlaneTimes{ { 193, 255 } });
+    g.zc = (N + n - 1) / n;
+    g.items = g.tx * g.ty * ((N + g.zc - 1) / g.zc);
+    g.ctas = std::min(g.items, kDiagCtas<real> * device_sm_count());
+    return g;
+}
+
+template <typename real, typename IT>
+cudaError_t launch_diag_whole_it(const View<real> &v, int N, const DiagArgs &da, cudaStream_t st)
+{
+    constexpr size_t smem = DiagGeo::smem<real>;
+    constexpr int minb = kDiagCtas<real>;
+    static unsigned long long configured = 0;   // per device; dynamic plus static smem may pass 48 KB
+    const unsigned long long dev_bit = 1ULL << device_slot();
+    if (!(configured & dev_bit)) {
+        const cudaError_t e = cudaFuncSetAttribute(k_diag_whole<real, IT, minb>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        configured |= dev_bit;
+    }
+    const DiagGrid g = diag_whole_grid<real>(N);
+    k_diag_whole<real, IT, minb><<<g.ctas, 256, smem, st>>>(v, N, g.tx, g.ty, g.items, g.zc, df_from(da.dc.g_div),
+                                                           df_from(da.dc.g_phi), da);
+    return cudaGetLastError();
+}
+}  // namespace
+
+int fused_diag_max_ctas() { return std::max(kDiagCtas<float>, kDiagCtas<double>) * device_sm_count(); }
+
+template <typename real>
+cudaError_t launch_fused_diag(const View<real> &v, int N, const DiagArgs &da, cudaStream_t st)
+{
+    return (long long)N * N * N < (1LL << 31) ? launch_diag_whole_it<real, int>(v, N, da, st)
+                                              : launch_diag_whole_it<real, long long>(v, N, da, st);
+}
+
 template <typename real>
 cudaError_t launch_diag_whole(const View<real> &v, int N, const DiagCoef &c, DiagPartial *partials,
                               int capacity, DiagPartial *result, DiagList list, int fix_blocks, cudaStream_t st)
 {
     // one partial per CTA of the tile walk: refuse a buffer that cannot hold them
-    if (fused_diag_ctas(N) > capacity) return cudaErrorInvalidValue;
+    const int ctas = diag_whole_grid<real>(N).ctas;
+    if (ctas > capacity) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemsetAsync(list.count, 0, sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
     DiagArgs da;
@@ -416,7 +462,7 @@ cudaError_t launch_diag_whole(const View<real> &v, int N, const DiagCoef &c, Dia
     da.list = list;
     e = launch_fused_diag<real>(v, N, da, st);
     if (e != cudaSuccess) return e;
-    return launch_diag_reduce<real>(v, N, partials, fused_diag_ctas(N), result, list, fix_blocks, st);
+    return launch_diag_reduce<real>(v, N, partials, ctas, result, list, fix_blocks, st);
 }
 
 template <typename real>
@@ -442,13 +488,13 @@ cudaError_t launch_diag(const View<real> &v, int N, Box b, const DiagCoef &c, Di
 {
     if (exact) {
         k_diag_exact<real><<<nblocks, NT, 0, st>>>(v, N, b, c, partials);
-        k_diag_finish<<<1, 32, 0, st>>>(partials, nblocks, result);
+        k_diag_sum<<<1, 1024, 0, st>>>(partials, nblocks, result);
         return cudaGetLastError();
     }
     cudaError_t e = cudaMemsetAsync(list.count, 0, sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
     k_diag_fast<real><<<nblocks, NT, 0, st>>>(v, N, b, c, partials, list);
-    k_diag_finish<<<1, 32, 0, st>>>(partials, nblocks, result);
+    k_diag_sum<<<1, 1024, 0, st>>>(partials, nblocks, result);
     k_diag_fixup<real><<<nblocks, 128, 0, st>>>(v, N, list, result);
     return cudaGetLastError();
 }
@@ -599,12 +645,17 @@ extern "C" ah_status ah_observables_noalloc(const float *const fields[10], int32
     list.capacity = kNoAllocListCap;
     DiagPartial *result = reinterpret_cast<DiagPartial *>(d_sums);
     const int nblocks = std::min(diag_grid_blocks(sms), kNoAllocBlocks);
-    const Box b{ 0, 0, 0, N, N, N };
-    const DiagCoef dc = host_diag_coef(*cfg, step);
+    DiagArgs da;
+    da.dc = host_diag_coef(*cfg, step);
+    da.partials = partials;
+    da.list = list;
+    const int ctas = diag_whole_grid<float>(N).ctas;
+    if (ctas > kNoAllocBlocks)
+        return host_fail(AH_ERR_CUDA, "ah_observables_noalloc: more resident CTAs than the scratch has partials");
     cudaError_t e = cudaMemsetAsync(list.count, 0, sizeof(unsigned long long), stream);
+    if (e == cudaSuccess) e = launch_fused_diag<float>(v, N, da, stream);
     if (e == cudaSuccess) {
-        k_diag_fast<float><<<nblocks, NT, 0, stream>>>(v, N, b, dc, partials, list);
-        k_diag_finish<<<1, 32, 0, stream>>>(partials, nblocks, result);
+        k_diag_sum<<<1, 1024, 0, stream>>>(partials, ctas, result);
         k_noalloc_fixup<float><<<nblocks, 128, 0, stream>>>(v, N, list, result);
         k_noalloc_wind_clear<<<1, 32, 0, stream>>>(list, result);
         k_noalloc_wind_all<float><<<nblocks, 256, 0, stream>>>(v, N, list, result);

@@ -19,16 +19,13 @@
 // state exactly once from DRAM; halo re-reads are served by L2.  Periodic
 // boundaries are applied in the index arithmetic.
 //
-// The same tile walk serves three kernels: k_fused (one lattice, one step),
-// k_fused_batch (persistent CTAs over the tiles of many lattices) and, in
-// MODE_DIAG, k_fused_diag (the whole-lattice diagnostics of Sec. 2: energy
-// sums, Gauss residual and plaquette windings of the current state, nothing
-// written back).  The shapes (tile height, sites per thread in x, resident
+// The same tile walk serves two kernels: k_fused (one lattice, one step) and
+// k_fused_batch (persistent CTAs over the tiles of many lattices).  FP64
+// lattices of the default shape run step_tile.cuh instead.  The shapes (tile height, sites per thread in x, resident
 // CTAs per SM) and the number of z chunks per column are chosen by the
 // autotuner; a chunk count that fills the last wave of CTAs matters because
 // each CTA marches a whole chunk.
 #include "ah_internal.cuh"
-#include "diag_common.cuh"
 #include "sincos32.cuh"
 #include "fused_common.cuh"
 #include "step_tile.cuh"
@@ -36,19 +33,14 @@
 namespace ah {
 namespace {
 
-// Kernel modes: the step, or the diagnostics of the current state (the same
-// tile walk with nothing written back).
-enum { MODE_STEP = 0, MODE_DIAG = 1 };
-
 // Each thread owns RX consecutive sites in x times RY rows (y stride 8).
 // One work item of the fused step: tile (bx, by) of plane chunk bz, marched in z.
 
 // IT: site-index type (int when N^3 < 2^31, so every field address is one
 // 32 x 32 -> 64-bit multiply-add; long long otherwise).
-template <typename real, int TY, int RX, typename IT, int MODE = MODE_STEP>
+template <typename real, int TY, int RX, typename IT>
 __device__ __forceinline__ void fused_tile(const View<real> &v, int N, int zc, const KickCoef<real> &c,
-                                           int bx, int by, int bz, unsigned char *smem_raw,
-                                           const DiagArgs *da = nullptr)
+                                           int bx, int by, int bz, unsigned char *smem_raw)
 {
     using G = Geo<real, TY, RX>;
     using IO = Row<real, RX>;
@@ -56,60 +48,11 @@ __device__ __forceinline__ void fused_tile(const View<real> &v, int N, int zc, c
     cpx<real> *sU = reinterpret_cast<cpx<real> *>(smem_raw);   // [2 planes][3 dirs][NE]
     cpx<real> *sF = sU + 2 * 3 * NE;                            // [2 planes][NE] phi
     real *sP = reinterpret_cast<real *>(sF + 2 * NE);           // [3][NP] sin Xi_12, _13, _23
-    C2<real> *sE = reinterpret_cast<C2<real> *>(smem_raw + G::diag_off);   // MODE_DIAG: [3][NE] edges
 
     const int tid = threadIdx.x, lx = tid & 31, wy = tid >> 5;
     const int x0 = bx * TX, y0 = by * TY;
     const int z0 = bz * zc;
-    constexpr bool STEP = MODE == MODE_STEP, DIAG = MODE == MODE_DIAG;
-    // per-thread diagnostic accumulators (MODE_DIAG): the energy sums of
-    // ah_obs 3..13 (compensated, state precision; 0..2 follow from 3..7), the
-    // Gauss residual sums and max (FP64), max |theta|, winding counters,
-    // non-finite sites
-    Acc<real> dacc[14];
-    real dtmax = real(0);
-    int dic[kNumInt] = { 0, 0, 0, 0, 0, 0, 0, 0 };   // per thread at most 3 x 2048 planes x |W| <= 2
-    // Gauss residual G = g_div div E + g_phi Im(conj(phi) Pi): FP64 for FP64
-    // data; for FP32 data in double-float arithmetic (each G to about 2^-44 of
-    // |g_div div E| + |g_phi Im(conj(phi) Pi)|), G^2 and that scale^2 summed
-    // with compensation after scaling by 2^60, max |G| kept as a double-float
-    double dg2 = 0.0, dgs2 = 0.0, dgmax = 0.0;
-    Acc<float> fg2, fgs2;
-    DF fgmax{ 0.f, 0.f };
-    DF cg_div{ 0.f, 0.f }, cg_phi{ 0.f, 0.f };
-    real k_inv_dx2 = 0, k_v = 0, k_eel = 0, k_b = 0, k_sig2 = 0;
-    if constexpr (DIAG) {
-        const DiagCoef &dc = da->dc;
-        cg_div = df_from(dc.g_div);
-        cg_phi = df_from(dc.g_phi);
-        k_inv_dx2 = (real)dc.inv_dx2; k_v = (real)dc.v_coef; k_eel = (real)dc.eel_coef;
-        k_b = (real)dc.b_coef; k_sig2 = (real)dc.sigma2;
-    }
-    auto diag_flush = [&]() {
-        if constexpr (DIAG) {
-            double accd[kNumSums];
-#pragma unroll
-            for (int k = 3; k < 14; ++k) accd[k] = dacc[k].value();
-            // the sums of L, rho and p are linear in those of K, G2, V, E_el, B
-            accd[0] = accd[3] - accd[4] - accd[5] + accd[6] - accd[7];
-            accd[1] = accd[3] + accd[4] + accd[5] + accd[6] + accd[7];
-            accd[2] = accd[3] - accd[4] * (1.0 / 3.0) - accd[5] + (accd[6] + accd[7]) * (1.0 / 3.0);
-            if constexpr (sizeof(real) == 4) {
-                dg2 = fg2.value() * 0x1p-60;
-                dgs2 = fgs2.value() * 0x1p-60;
-                dgmax = (double)fgmax.h + (double)fgmax.l;
-            }
-            accd[14] = dg2;
-            accd[15] = dgs2;
-            double mx[kNumMax] = { dgmax, (double)dtmax };
-            const int cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-            long long dil[kNumInt];
-#pragma unroll
-            for (int k = 0; k < kNumInt; ++k) dil[k] = dic[k];
-            block_reduce<256>(accd, mx, dil, &da->partials[cta]);
-        }
-    };
-    if (z0 >= N) { diag_flush(); return; }
+    if (z0 >= N) return;
     const int z1 = min(z0 + zc, N);
     const IT NN = (IT)N * (IT)N;
 
@@ -187,22 +130,6 @@ __device__ __forceinline__ void fused_tile(const View<real> &v, int N, int zc, c
     // own-site registers carried along z
     cpx<real> ph_m[NS], ph_0[NS], u3_m[NS];
     real th_0[NS][3], p13_m[NS], p23_m[NS];
-    real e3_m[NS];                           // MODE_DIAG: E_3 of plane z-1
-    // MODE_DIAG: scaled edge products conj(phi^x) U_d^x phi^{x+d} of the own
-    // sites for d = 1, 2 in plane z (computed one plane ahead) and d = 3
-    using Z = C2<real>;
-    Z ed1[NS], ed2[NS], ed3[NS];
-    auto zc_ = [](cpx<real> a) { return Z{ a.r, a.i }; };
-    auto edge = [&](cpx<real> fa, cpx<real> u, cpx<real> fb) {
-        Z z = cmul(conj(zc_(fa)), cmul(zc_(u), zc_(fb)));
-        unit_scale_or_nan(z);
-        return z;
-    };
-    if constexpr (DIAG) {
-        const IT base = (IT)(z0 == 0 ? N - 1 : z0 - 1) * NN;
-#pragma unroll
-        for (int m = 0; m < NS; ++m) e3_m[m] = v.e3[base + (IT)roff[m / RX] + (IT)(m % RX)];
-    }
 
     // prologue: planes z0-1 and z0
     // ring slot of plane z: (z - z0 + 1) & 1
@@ -227,11 +154,6 @@ __device__ __forceinline__ void fused_tile(const View<real> &v, int N, int zc, c
         u3_m[m] = Um[2 * NE + e];
         p13_m[m] = plaq(Um[e], Um[2 * NE + e + 1], U0[e], Um[2 * NE + e]);
         p23_m[m] = plaq(Um[NE + e], Um[2 * NE + e + EX], U0[NE + e], Um[2 * NE + e]);
-        if constexpr (DIAG) {
-            const cpx<real> *F0p = sF + b0 * NE;
-            ed1[m] = edge(F0p[e], U0[e], F0p[e + 1]);
-            ed2[m] = edge(F0p[e], U0[NE + e], F0p[e + EX]);
-        }
     }
     __syncthreads();
 
@@ -265,74 +187,24 @@ __device__ __forceinline__ void fused_tile(const View<real> &v, int N, int zc, c
         // B: plaquette sines of plane z on the tile (own sites) and its low halos
         const cpx<real> *U0 = sU + bc * 3 * NE, *U1p = sU + bn * 3 * NE;
         real p12[NS], p13[NS], p23[NS];
-        [[maybe_unused]] Z ez1[NS], ez2[NS];      // MODE_DIAG: own d = 1, 2 edges of plane z+1
-        // MODE_DIAG: a plaquette whose four edges all have |Arg| < pi/4 has
-        // W = 0; when every edge that the CTA's plaquettes of plane z use passes
-        // that test (smooth regions), the carry chains are skipped
-        [[maybe_unused]] bool own_smooth = true;
-        [[maybe_unused]] auto smooth1 = [](const Z &z) { return z.r > real(1.001) * fabs(z.i); };
-        [[maybe_unused]] real bcos[NS];          // MODE_DIAG: 1 - cos Xi summed over the three orientations
 #pragma unroll
         for (int m = 0; m < NS; ++m) {
             const int e = eix(m), p = pix(m);
-            if constexpr (DIAG) {
-                const cpx<real> x12 = plaq2(U0[e], U0[NE + e + 1], U0[e + EX], U0[NE + e]);
-                const cpx<real> x13 = plaq2(U0[e], U0[2 * NE + e + 1], U1p[e], U0[2 * NE + e]);
-                const cpx<real> x23 = plaq2(U0[NE + e], U0[2 * NE + e + EX], U1p[NE + e], U0[2 * NE + e]);
-                p12[m] = x12.i; p13[m] = x13.i; p23[m] = x23.i;
-                bcos[m] = one_minus_cos(x12.r, x12.i) + one_minus_cos(x13.r, x13.i) +
-                          one_minus_cos(x23.r, x23.i);
-            } else {
-                p12[m] = plaq(U0[e], U0[NE + e + 1], U0[e + EX], U0[NE + e]);
-                p13[m] = plaq(U0[e], U0[2 * NE + e + 1], U1p[e], U0[2 * NE + e]);
-                p23[m] = plaq(U0[NE + e], U0[2 * NE + e + EX], U1p[NE + e], U0[2 * NE + e]);
-            }
-            if constexpr (STEP) {              // the sines feed only the E kick
-                sP[p] = p12[m];
-                sP[G::NP + p] = p13[m];
-                sP[2 * G::NP + p] = p23[m];
-            }
+            p12[m] = plaq(U0[e], U0[NE + e + 1], U0[e + EX], U0[NE + e]);
+            p13[m] = plaq(U0[e], U0[2 * NE + e + 1], U1p[e], U0[2 * NE + e]);
+            p23[m] = plaq(U0[NE + e], U0[2 * NE + e + EX], U1p[NE + e], U0[2 * NE + e]);
+            sP[p] = p12[m];
+            sP[G::NP + p] = p13[m];
+            sP[2 * G::NP + p] = p23[m];
         }
-        if constexpr (DIAG) {
-            // own edges of plane z, then the right column's d = 2, 3 and the
-            // top row's d = 1, 3 edges that the tile's last column / row need
-            const cpx<real> *F0 = sF + bc * NE, *F1 = sF + bn * NE;
-#pragma unroll
-            for (int m = 0; m < NS; ++m) {
-                const int e = eix(m);
-                ed3[m] = edge(F0[e], U0[2 * NE + e], ph_p[m]);
-                ez1[m] = edge(F1[e], U1p[e], F1[e + 1]);
-                ez2[m] = edge(F1[e], U1p[NE + e], F1[e + EX]);
-                sE[e] = ed1[m];
-                sE[NE + e] = ed2[m];
-                sE[2 * NE + e] = ed3[m];
-                own_smooth = own_smooth && smooth1(ed1[m]) && smooth1(ed2[m]) && smooth1(ed3[m]) &&
-                             smooth1(ez1[m]) && smooth1(ez2[m]);
-            }
-            if (tid < TY) {
-                const int e = (tid + 1) * EX + EX - 1;
-                const Z a = edge(F0[e], U0[NE + e], F0[e + EX]), b = edge(F0[e], U0[2 * NE + e], F1[e]);
-                sE[NE + e] = a;
-                sE[2 * NE + e] = b;
-                own_smooth = own_smooth && smooth1(a) && smooth1(b);
-            } else if (tid < TY + TX) {
-                const int e = (EY - 1) * EX + tid - TY + 1;
-                const Z a = edge(F0[e], U0[e], F0[e + 1]), b = edge(F0[e], U0[2 * NE + e], F1[e]);
-                sE[e] = a;
-                sE[2 * NE + e] = b;
-                own_smooth = own_smooth && smooth1(a) && smooth1(b);
-            }
-        }
-        if (STEP && tid < G::NPHALO) {
+        if (tid < G::NPHALO) {
             const int px = tid < PX ? tid : 0, py = tid < PX ? 0 : tid - PX + 1;
             const int e = py * EX + px, p = py * PX + px;
             sP[p] = plaq(U0[e], U0[NE + e + 1], U0[e + EX], U0[NE + e]);
             sP[G::NP + p] = plaq(U0[e], U0[2 * NE + e + 1], U1p[e], U0[2 * NE + e]);
             sP[2 * G::NP + p] = plaq(U0[NE + e], U0[2 * NE + e + EX], U1p[NE + e], U0[2 * NE + e]);
         }
-        [[maybe_unused]] bool smooth_cta = false;
-        if constexpr (DIAG) smooth_cta = __syncthreads_and(own_smooth) != 0;
-        else __syncthreads();
+        __syncthreads();
 
         // C: kicks and drifts of the own sites of plane z
         const cpx<real> *F0 = sF + bc * NE;
@@ -365,82 +237,6 @@ __device__ __forceinline__ void fused_tile(const View<real> &v, int N, int zc, c
             const real ne1 = c.c_edamp * e1[m] + c.c_cur * cu1 - c.c_curl * cl1;
             const real ne2 = c.c_edamp * e2[m] + c.c_cur * cu2 - c.c_curl * cl2;
             const real ne3 = c.c_edamp * e3[m] + c.c_cur * cu3 - c.c_curl * cl3;
-            if constexpr (DIAG) if (wr[m / RX]) {
-                const real K = pr[m] * pr[m] + pim[m] * pim[m];
-                const real d1r = w1.r - f0.r, d1i = w1.i - f0.i, d2r = w2.r - f0.r, d2i = w2.i - f0.i;
-                const real d3r = w3.r - f0.r, d3i = w3.i - f0.i;
-                const real G2 = (d1r * d1r + d1i * d1i + d2r * d2r + d2i * d2i + d3r * d3r + d3i * d3i) *
-                                k_inv_dx2;
-                const real m2 = f0.r * f0.r + f0.i * f0.i - k_sig2;
-                const real V = k_v * m2 * m2;
-                const real Eel = k_eel * (e1[m] * e1[m] + e2[m] * e2[m] + e3[m] * e3[m]);
-                const real B = k_b * bcos[m];
-                const real L = K - G2 - V + Eel - B;
-                const real rho = K + G2 + V + Eel + B;
-                const real pp = K - G2 * real(1.0 / 3.0) - V + (Eel + B) * real(1.0 / 3.0);
-                dacc[3].add(K); dacc[4].add(G2);
-                dacc[5].add(V); dacc[6].add(Eel); dacc[7].add(B); dacc[8].add(K * V); dacc[9].add(G2 * V);
-                dacc[10].add(K * L); dacc[11].add(G2 * L); dacc[12].add(pp * L); dacc[13].add(rho * L);
-                dtmax = fmax(dtmax, fmax(fabs(th_0[m][0]), fmax(fabs(th_0[m][1]), fabs(th_0[m][2]))));
-                dic[7] += !(isfinite(L) && isfinite(rho) && isfinite(pp));
-                const int my = m / RX, mx = m % RX;
-                const int gx = x0 + RX * lx + mx, gy = y0 + wy + 8 * my;
-                // Gauss residual (nothing is written in this mode, so the
-                // backward neighbours' E are the current ones)
-                {
-                    const IT s = base + (IT)roff[my] + (IT)mx;
-                    const real e1b = v.e1[gx == 0 ? s + (IT)(N - 1) : s - 1];
-                    const real e2b = v.e2[gy == 0 ? s + (NN - (IT)N) : s - (IT)N];
-                    if constexpr (sizeof(real) == 8) {
-                        const DiagCoef &dc = da->dc;
-                        const double div = (e1[m] - e1b) + (e2[m] - e2b) + (e3[m] - e3_m[m]);
-                        const double g1 = dc.g_div * div;
-                        const double g2 = dc.g_phi * (f0.r * pim[m] - f0.i * pr[m]);
-                        const double Gs = g1 + g2, gs = fabs(g1) + fabs(g2);
-                        dg2 += Gs * Gs;
-                        dgs2 += gs * gs;
-                        dgmax = fmax(dgmax, fabs(Gs));
-                    } else {
-                        // differences and products of FP32 values are exact as pairs
-                        const DF div = df_add(df_add(two_sum(e1[m], -e1b), two_sum(e2[m], -e2b)),
-                                              two_sum(e3[m], -e3_m[m]));
-                        const DF a = two_prod(f0.r, pim[m]), b = two_prod(f0.i, pr[m]);
-                        const DF g1 = df_mul(cg_div, div), g2 = df_mul(cg_phi, df_add(a, { -b.h, -b.l }));
-                        DF Gs = df_add(g1, g2);
-                        if (Gs.h < 0.f) Gs = { -Gs.h, -Gs.l };
-                        const float gs = fabsf(g1.h) + fabsf(g2.h);
-                        const float sg = Gs.h * 0x1p30f, ss = gs * 0x1p30f;
-                        fg2.add(sg * sg);
-                        fgs2.add(ss * ss);
-                        if (Gs.h > fgmax.h || (Gs.h == fgmax.h && Gs.l > fgmax.l)) fgmax = Gs;
-                    }
-                }
-                // windings of the plaquettes (12), (13), (23) based at x (Eq. 9)
-                // from their twelve edge products conj(phi^a) U phi^b: the own
-                // ones (this plane and, for d = 1, 2, the next) and the x and y
-                // neighbours' from shared memory
-                const Z z2_1 = sE[NE + e + 1], z3_1 = sE[2 * NE + e + 1];
-                const Z z1_2 = sE[e + EX], z3_2 = sE[2 * NE + e + EX];
-                int wq[3] = { 0, 0, 0 };
-                if (!smooth_cta) {
-                    wq[0] = winding_scaled(ed1[m], z2_1, z1_2, ed2[m]);
-                    wq[1] = winding_scaled(ed1[m], z3_1, ez1[m], ed3[m]);
-                    wq[2] = winding_scaled(ed2[m], z3_2, ez2[m], ed3[m]);
-                }
-                const unsigned long long site =
-                    (unsigned long long)((long long)z * N * (long long)N + (long long)roff[my] + mx);
-#pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    if (wq[q] == INT_MIN) {
-                        const unsigned long long k = atomicAdd(da->list.count, 1ULL);
-                        if (k < (unsigned long long)da->list.capacity) da->list.items[k] = site * 4ULL + q;
-                    } else {
-                        dic[q] += wq[q] < 0 ? -wq[q] : wq[q];
-                        dic[3 + q] += wq[q];
-                        dic[6] += wq[q] != 0;
-                    }
-                }
-            }
             o_pr[m] = npr; o_pi[m] = npi;
             o_e1[m] = ne1; o_e2[m] = ne2; o_e3[m] = ne3;
             o_fr[m] = f0.r + c.dt * npr;
@@ -454,11 +250,6 @@ __device__ __forceinline__ void fused_tile(const View<real> &v, int N, int zc, c
                 o_t3[m] = wrap_phase(o_t3[m]);
             }
             // march: plane z becomes z-1
-            if constexpr (DIAG) {
-                e3_m[m] = e3[m];
-                ed1[m] = ez1[m];
-                ed2[m] = ez2[m];
-            }
             ph_m[m] = f0;
             u3_m[m] = u3;
             p13_m[m] = q13;
@@ -468,7 +259,7 @@ __device__ __forceinline__ void fused_tile(const View<real> &v, int N, int zc, c
         }
 #pragma unroll
         for (int my = 0; my < RY; ++my) {
-            if (STEP && wr[my]) {
+            if (wr[my]) {
                 const IT s = base + (IT)roff[my];
                 const int k = my * RX;
                 IO::st(v.pir + s, o_pr + k); IO::st(v.pii + s, o_pi + k);
@@ -483,7 +274,6 @@ __device__ __forceinline__ void fused_tile(const View<real> &v, int N, int zc, c
         plane_step(z0 + k, IC<1>{});
         if (z0 + k + 1 < z1) plane_step(z0 + k + 1, IC<0>{});
     }
-    diag_flush();
 }
 
 // Shapes that run step_tile instead of fused_tile: FP64, one site per thread.
@@ -501,16 +291,6 @@ __global__ void __launch_bounds__(256, MINB) k_fused(View<real> v, int N, int zc
         step_tile<real, TY, IT>(v, N, zc, c, blockIdx.x, blockIdx.y, blockIdx.z, smem_raw);
     else
         fused_tile<real, TY, RX, IT>(v, N, zc, c, blockIdx.x, blockIdx.y, blockIdx.z, smem_raw);
-}
-
-// Diagnostics of the current state through the step's tile walk (tile 32 x 8,
-// nothing written back); one DiagPartial per CTA.
-template <typename real, typename IT>
-__global__ void __launch_bounds__(256) k_fused_diag(View<real> v, int N, int zc, DiagArgs da)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const KickCoef<real> c{};
-    fused_tile<real, 8, 1, IT, MODE_DIAG>(v, N, zc, c, blockIdx.x, blockIdx.y, blockIdx.z, smem_raw, &da);
 }
 
 // Batched fused step: persistent CTAs take (lattice, tile) work items from a
@@ -723,52 +503,6 @@ cudaError_t launch_fused_step<double>(const View<double> &v, int N, const KickCo
     }
 }
 
-
-// ---- diagnostics through the fused tile ----
-namespace {
-template <typename real, typename IT>
-cudaError_t launch_diag_it(const View<real> &v, int N, const DiagArgs &da, cudaStream_t st)
-{
-    using G = Geo<real, 8, 1>;
-    static unsigned long long configured = 0;   // per device; dynamic plus static smem may pass 48 KB
-    const unsigned long long dev_bit = 1ULL << device_slot();
-    if (!(configured & dev_bit)) {
-        const cudaError_t e = cudaFuncSetAttribute(k_fused_diag<real, IT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)G::smem_diag);
-        if (e != cudaSuccess) return e;
-        configured |= dev_bit;
-    }
-    int tx, ty, nch, zc;
-    fused_diag_grid(N, &tx, &ty, &nch, &zc);
-    k_fused_diag<real, IT><<<dim3(tx, ty, nch), 256, G::smem_diag, st>>>(v, N, zc, da);
-    return cudaGetLastError();
-}
-}  // namespace
-
-void fused_diag_grid(int N, int *tx, int *ty, int *nch, int *zc)
-{
-    *tx = (N + 31) / 32;
-    *ty = (N + 7) / 8;
-    const int n = choose_chunks(N, (long long)*tx * *ty, 2, 4, PlaneTimes{ { 255, 255 } });   // 2 CTAs / SM
-    *zc = (N + n - 1) / n;
-    *nch = (N + *zc - 1) / *zc;
-}
-
-int fused_diag_ctas(int N)
-{
-    int tx, ty, nch, zc;
-    fused_diag_grid(N, &tx, &ty, &nch, &zc);
-    return tx * ty * nch;
-}
-
-template <typename real>
-cudaError_t launch_fused_diag(const View<real> &v, int N, const DiagArgs &da, cudaStream_t st)
-{
-    return (long long)N * N * N < (1LL << 31) ? launch_diag_it<real, int>(v, N, da, st)
-                                              : launch_diag_it<real, long long>(v, N, da, st);
-}
-template cudaError_t launch_fused_diag<float>(const View<float> &, int, const DiagArgs &, cudaStream_t);
-template cudaError_t launch_fused_diag<double>(const View<double> &, int, const DiagArgs &, cudaStream_t);
 
 // ---- batched step ----
 namespace {
