@@ -58,56 +58,79 @@ __device__ __forceinline__ float site_phase(float r, float i)
     return hi > 1e-30f && hi < 1e30f && lo >= 0.f ? a : __int_as_float(0x7fc00000);
 }
 
-// n of one link and whether its bracket is too near the cut; k: whole turns
-// already taken from theta
+// n of a link whose bracket is a - 2 pi n, and whether the bracket is too near
+// the cut: adding 1.5 x 2^23 rounds to the nearest integer, which the low bits then
+// hold.
+constexpr float kRound = 12582912.0f;
+constexpr int kRoundBits = 0x4b400000;
 __device__ __forceinline__ int turns(float a, bool *cut)
 {
-    const float k = rintf(a * kInvTwoPi32);
+    const float kb = __fmaf_rn(a, kInvTwoPi32, kRound), k = __fsub_rn(kb, kRound);
     *cut = !(fabsf(fmaf(-k, kTwoPi32, a)) <= kPi32 - kCutMargin);
-    return (int)k;
+    return __float_as_int(kb) - kRoundBits;
 }
-// n_1, n_2, n_3 as 9-bit fields and their cut flags; links with more than 255
-// turns count as near the cut
-struct LinkTurns { int n; bool cut; };
-__device__ __forceinline__ LinkTurns link_turns(float a, float b, float theta)
+// n_1, n_2, n_3 of a site's links to neighbours of phase b[], and a bit for each
+// that is too near the cut.  Phases past 8 give up their whole turns first, and
+// links with more than 24 turns count as near the cut, so that sums of four fit
+// the 8-bit fields below.
+__device__ __forceinline__ int link_turns(float a, const float b[3], const float t[3], int n[3])
 {
-    LinkTurns t;
-    if (fabsf(theta) <= 8.f) {
-        t.n = turns(b - a + theta, &t.cut);
+    const float m = fmaxf(fabsf(t[0]), fmaxf(fabsf(t[1]), fabsf(t[2])));
+    bool c[3];
+    if (__all_sync(__activemask(), m <= 8.f)) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) n[d] = turns(b[d] - a + t[d], &c[d]);
     } else {
-        // whole turns out of a large phase first
-        const float k = rintf(theta * kInvTwoPi32);
-        const float r = fmaf(k, 1.74845553e-7f, fmaf(-k, 6.28318548f, theta));
-        t.n = turns(b - a + r, &t.cut);
-        t.cut = t.cut || !(fabsf(k) < 250.f);
-        t.n += t.cut ? 0 : (int)k;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const float k = rintf(t[d] * kInvTwoPi32);
+            const float r = fmaf(k, 1.74845553e-7f, fmaf(-k, 6.28318548f, t[d]));
+            n[d] = turns(b[d] - a + r, &c[d]);
+            c[d] = c[d] || !(fabsf(k) <= 24.f);
+            n[d] = c[d] ? 0 : n[d] + (int)k;
+        }
     }
-    if (t.cut) t.n = 0;
-    return t;
+    if (!__any_sync(__activemask(), c[0] | c[1] | c[2])) return 0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) n[d] = c[d] ? 0 : n[d];
+    return (int)c[0] | (int)c[1] << 1 | (int)c[2] << 2;
 }
-__device__ __forceinline__ unsigned pack_turns(LinkTurns a, LinkTurns b, LinkTurns c)
+// The terms that a link's n adds to n_1 + n_2 - n_3 - n_4 of the plaquettes (12),
+// (13), (23), as three 8-bit fields (modulo 2^24) under three cut bits: of a site's
+// own links, of its links seen from x - 1 and from x - y, and from z - 1.  Words are
+// added, cut bits or-ed.
+__device__ __forceinline__ unsigned field_word(int v, int cut) { return ((unsigned)v & 0xffffffu) | (unsigned)cut << 24; }
+__device__ __forceinline__ unsigned own_word(const int n[3], int c)
 {
-    return (unsigned)((a.n & 511) | (b.n & 511) << 9 | (c.n & 511) << 18) | (unsigned)a.cut << 27 |
-           (unsigned)b.cut << 28 | (unsigned)c.cut << 29;
+    const int v = n[0] * 257 + n[1] * 65535 - n[2] * 65792;
+    return field_word(v, c ? ((c | c >> 1) & 1) | ((c | c >> 2) & 1) << 1 | ((c >> 1 | c >> 2) & 1) << 2 : 0);
 }
-__device__ __forceinline__ int turn_of(unsigned w, int d) { return (int)(w << (23 - 9 * d)) >> 23; }
-__device__ __forceinline__ bool cut_of(unsigned w, int d) { return (w >> (27 + d)) & 1u; }
+__device__ __forceinline__ unsigned x_word(int n2, int n3, int c)
+{
+    return field_word(n2 + n3 * 256, c ? (c >> 1 & 1) | (c >> 2 & 1) << 1 : 0);
+}
+__device__ __forceinline__ unsigned y_word(int n1, int n3, int c)
+{
+    return field_word(n3 * 65536 - n1, c ? (c & 1) | (c >> 2 & 1) << 2 : 0);
+}
+__device__ __forceinline__ unsigned z_word(const int n[3], int c)
+{
+    return field_word(-n[0] * 256 - n[1] * 65536, c ? (c & 1) << 1 | (c >> 1 & 1) << 2 : 0);
+}
 
-// 1 - cos Xi summed over the three plaquettes of a site, the whole turns N of each
-// and the plaquettes whose [Xi] is too near the cut, from the four phases of each
-// (as in Eq. 3: ti, tj at x, tij = theta_i^{x+j}, tji = theta_j^{x+i})
-struct XiTerms { int n[3]; int cut; };
+// 1 - cos Xi summed over the three plaquettes of a site, from the four phases of
+// each (as in Eq. 3: ti, tj at x, tij = theta_i^{x+j}, tji = theta_j^{x+i}); *word
+// the whole turns -N of each and the plaquettes whose [Xi] is too near the cut
 __device__ __forceinline__ float xi_terms(const float *ti, const float *tij, const float *tj, const float *tji,
-                                          XiTerms *o)
+                                          unsigned *word)
 {
     float x[3], m = 0.f, sum = 0.f;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         x[k] = (ti[k] - tij[k]) + (tji[k] - tj[k]);
         m = fmaxf(m, fabsf(x[k]));
-        o->n[k] = 0;
     }
-    o->cut = 0;
+    *word = 0;
     if (__all_sync(__activemask(), m <= 0.78f)) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
@@ -119,6 +142,7 @@ __device__ __forceinline__ float xi_terms(const float *ti, const float *tij, con
         }
         return sum;
     }
+    int n = 0, cuts = 0;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const DF d1 = two_sum(ti[k], -tij[k]), d2 = two_sum(tji[k], -tj[k]), d3 = two_sum(d1.h, d2.h);
@@ -126,17 +150,18 @@ __device__ __forceinline__ float xi_terms(const float *ti, const float *tij, con
         const float kf = rintf(d3.h * kInvTwoPi32);
         // [Xi] = Xi - 2 pi k with 2 pi in two parts
         const float r = fmaf(kf, 1.74845553e-7f, fmaf(-kf, 6.28318548f, d3.h)) + lo;
-        const bool cut = !(fabsf(r) <= kPi32 - kCutMargin) || !(fabsf(kf) < 1e6f);
-        o->cut |= cut << k;
-        o->n[k] = cut ? 0 : (int)kf;
+        const bool cut = !(fabsf(r) <= kPi32 - kCutMargin) || !(fabsf(kf) <= 96.f);
+        cuts |= cut << k;
+        n -= cut ? 0 : (int)kf << 8 * k;
         float s, c;
         sincos_link(0.5f * r, &s, &c);
         sum = fmaf(2.f * s, s, sum);
     }
+    *word = field_word(n, cuts);
     return sum;
 }
 __device__ __forceinline__ double xi_terms(const double *ti, const double *tij, const double *tj, const double *tji,
-                                           XiTerms *o)
+                                           unsigned *word)
 {
     double x[3], sum = 0.0;
     int m = 0;
@@ -144,26 +169,27 @@ __device__ __forceinline__ double xi_terms(const double *ti, const double *tij, 
     for (int k = 0; k < 3; ++k) {
         x[k] = (ti[k] - tij[k]) + (tji[k] - tj[k]);
         m = max(m, abs_hi(x[k]));
-        o->n[k] = 0;
     }
-    o->cut = 0;
+    *word = 0;
     const unsigned mm = __reduce_max_sync(__activemask(), (unsigned)m);
     if (mm <= kHi04) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) sum += mm <= kHi2m4 ? vers_range<0>(x[k]) : vers_range<1>(x[k]);
         return sum;
     }
+    int n = 0, cuts = 0;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const float xf = (float)x[k], kf = rintf(xf * kInvTwoPi32);
         const float r = fmaf(kf, 1.74845553e-7f, fmaf(-kf, 6.28318548f, xf));
-        const bool cut = !(fabsf(r) <= kPi32 - kCutMargin - 1e-6f * fabsf(kf)) || !(fabsf(kf) < 1e2f);
-        o->cut |= cut << k;
-        o->n[k] = cut ? 0 : (int)kf;
+        const bool cut = !(fabsf(r) <= kPi32 - kCutMargin - 1e-6f * fabsf(kf)) || !(fabsf(kf) <= 96.f);
+        cuts |= cut << k;
+        n -= cut ? 0 : (int)kf << 8 * k;
         double s, c;
         sincos_reduced(0.5 * x[k], 0.0, &s, &c);
         sum += 2.0 * s * s;
     }
+    *word = field_word(n, cuts);
     return sum;
 }
 
@@ -182,11 +208,28 @@ __device__ __forceinline__ void diag_links(const double t[3], double s[3], doubl
 template <typename real> struct alignas(16) D4 { real a, b, c, d; };
 template <typename real> struct alignas(2 * sizeof(real)) D2 { real a, b; };
 
+// DiagCoef in the state precision (the Gauss coefficients of an FP32 state as
+// double-float pairs), converted once on the host: conversions from FP64 in the
+// kernel took a third of the FP64 pipe.
+template <typename real> struct SiteCoef;
+template <> struct SiteCoef<float> { float inv_dx2, v_coef, eel_coef, b_coef, sigma2; DF g_div, g_phi; };
+struct D1 { double h; };
+template <> struct SiteCoef<double> { double inv_dx2, v_coef, eel_coef, b_coef, sigma2; D1 g_div, g_phi; };
+inline SiteCoef<float> site_coef(const DiagCoef &d, float)
+{
+    return { (float)d.inv_dx2, (float)d.v_coef, (float)d.eel_coef, (float)d.b_coef, (float)d.sigma2, df_from(d.g_div),
+             df_from(d.g_phi) };
+}
+inline SiteCoef<double> site_coef(const DiagCoef &d, double)
+{
+    return { d.inv_dx2, d.v_coef, d.eel_coef, d.b_coef, d.sigma2, { d.g_div }, { d.g_phi } };
+}
+
 struct DiagGeo {
     static constexpr int TX = 32, TY = 8, NT = 256, EX = TX + 2, NE = EX * (TY + 2);
     // two copies of: { phi.re, phi.im, theta_3, theta_2 }, { E_1, E_2 }, theta_1,
-    // alpha, packed turns
-    template <typename real> static constexpr int bytes = NE * (7 * (int)sizeof(real) + 8);
+    // alpha, turns as seen from x - 1 and from x - y
+    template <typename real> static constexpr int bytes = NE * (7 * (int)sizeof(real) + 12);
     template <typename real> static constexpr size_t smem = 2 * (size_t)((bytes<real> + 15) / 16 * 16);
 };
 
@@ -203,7 +246,7 @@ struct DiagTile {
     int ic[kNumInt] = { 0, 0, 0, 0, 0, 0, 0, 0 };
 
     // one column of tiles: planes [z0, z1) of the 32 x 8 sites at (x0, y0)
-    __device__ __forceinline__ void column(const View<real> &v, int N, const DiagArgs &da, DF g_div, DF g_phi, int x0,
+    __device__ __forceinline__ void column(const View<real> &v, int N, const DiagArgs &da, const SiteCoef<real> &sc, int x0,
                                            int y0, int z0, int z1, unsigned char *smem)
     {
         const int lx = threadIdx.x & 31, wy = threadIdx.x >> 5;
@@ -223,9 +266,9 @@ struct DiagTile {
         const int half = (G::bytes<real> + 15) / 16 * 16;
         auto at4 = [&](int b) { return reinterpret_cast<D4<real> *>(smem + b * half); };
         auto at2 = [&](int b) { return reinterpret_cast<D2<real> *>(smem + b * half + NE * 4 * sizeof(real)); };
-        auto at1 = [&](int b) { return reinterpret_cast<real *>(smem + b * half + NE * 6 * sizeof(real)); };
-        auto atf = [&](int b) { return reinterpret_cast<float *>(smem + b * half + NE * 7 * sizeof(real)); };
-        auto atw = [&](int b) { return reinterpret_cast<unsigned *>(smem + b * half + NE * (7 * sizeof(real) + 4)); };
+        auto atw = [&](int b) { return reinterpret_cast<uint2 *>(smem + b * half + NE * 6 * sizeof(real)); };
+        auto at1 = [&](int b) { return reinterpret_cast<real *>(smem + b * half + NE * (6 * sizeof(real) + 8)); };
+        auto atf = [&](int b) { return reinterpret_cast<float *>(smem + b * half + NE * (7 * sizeof(real) + 8)); };
         auto wrapz = [&](int z) { return (IT)(z < 0 ? z + N : (z >= N ? z - N : z)) * NN; };
 
         // fields of the next plane, momenta of the current one
@@ -253,8 +296,7 @@ struct DiagTile {
         load_momenta(z0);
         a0 = site_phase((float)nf[0], (float)nf[1]);
         ra = fwd ? site_phase((float)rf[0], (float)rf[1]) : 0.f;
-        unsigned wm = 0;                         // own turns of plane z - 1
-        XiTerms xm{ { 0, 0, 0 }, 0 };
+        unsigned wm = 0;                         // own turns and N of plane z - 1
         for (int z = z0; z <= z1; ++z) {
             const int b = z & 1;
             f0[0] = nf[0]; f0[1] = nf[1];
@@ -283,73 +325,70 @@ struct DiagTile {
             const real e1x = at2(b)[e - 1].a, e2y = at2(b)[e - EX].b;
             if (z + 1 < z1) load_momenta(z + 1);
             const float an = z < z1 ? site_phase((float)nf[0], (float)nf[1]) : 0.f;
-            const LinkTurns n1 = link_turns(a0, ax, (float)t0[0]), n2 = link_turns(a0, ay, (float)t0[1]);
-            const LinkTurns n3 = link_turns(a0, an, (float)t0[2]);
-            const unsigned w = pack_turns(n1, n2, n3);
-            atw(b)[e] = w;
+            int n[3];
+            int nc;
+            {
+                const float bn[3] = { ax, ay, an }, tf[3] = { (float)t0[0], (float)t0[1], (float)t0[2] };
+                nc = link_turns(a0, bn, tf, n);
+                atw(b)[e] = make_uint2(x_word(n[1], n[2], nc), y_word(n[0], n[2], nc));
+            }
             if (fwd) {
                 // the row above: n_1, n_3; the column to the right: n_2, n_3
                 const float rn = z < z1 ? site_phase((float)rf[0], (float)rf[1]) : 0.f;
                 const float aj = above ? atf(b)[he + 1] : (lx < 8 ? atf(b)[he + EX] : 0.f);
-                const LinkTurns k = link_turns(ra, aj, (float)(above ? g0[0] : g0[1]));
-                atw(b)[he] = pack_turns(k, k, link_turns(ra, rn, (float)g0[2]));
+                const float bn[3] = { aj, aj, rn }, tf[3] = { (float)g0[0], (float)g0[1], (float)g0[2] };
+                int rk[3];
+                const int rc = link_turns(ra, bn, tf, rk);
+                atw(b)[he] = make_uint2(x_word(rk[1], rk[2], rc), y_word(rk[0], rk[2], rc));
                 ra = rn;
             }
             // windings of plane z - 1 (Eq. 9): its neighbours' turns are in the other copy
             if (z > z0 && own) {
-                const unsigned wx = atw(1 - b)[e + 1], wyv = atw(1 - b)[e + EX];
-                const int o1 = turn_of(wm, 0), o2 = turn_of(wm, 1), o3 = turn_of(wm, 2);
-                const int q12 = xm.n[0] - (o1 + turn_of(wx, 1) - turn_of(wyv, 0) - o2);
-                const int q13 = xm.n[1] - (o1 + turn_of(wx, 2) - n1.n - o3);
-                const int q23 = xm.n[2] - (o2 + turn_of(wyv, 2) - n2.n - o3);
-                const unsigned c1 = wm >> 27, cx = wx >> 27, cy = wyv >> 27;     // bits 0, 1, 2: links 1, 2, 3
-                const bool b12 = (c1 & 3) | (cx & 2) | (cy & 1) | (xm.cut & 1);
-                const bool b13 = (c1 & 5) | (cx & 4) | (unsigned)n1.cut | (xm.cut & 2);
-                const bool b23 = (c1 & 6) | (cy & 4) | (unsigned)n2.cut | (xm.cut & 4);
-                const int q[3] = { b12 ? 0 : q12, b13 ? 0 : q13, b23 ? 0 : q23 };
+                const unsigned wx = atw(1 - b)[e + 1].x, wyv = atw(1 - b)[e + EX].y, wz = z_word(n, nc);
+                const unsigned t = (0u - (wm + wx + wyv + wz)) & 0xffffffu, cuts = (wm | wx | wyv | wz) >> 24;
+                if (t | cuts) {
+                    const int w12 = (int)(t << 24) >> 24, r1 = ((int)(t << 8) >> 8) - w12 >> 8;
+                    const int w13 = (int)((unsigned)r1 << 24) >> 24, w23 = (int)((unsigned)(r1 - w13 >> 8) << 24) >> 24;
+                    const int q[3] = { w12, w13, w23 };
 #pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    ic[k] += abs(q[k]);
-                    ic[3 + k] += q[k];
-                    ic[6] += q[k] != 0;
-                }
-                if (b12 | b13 | b23) {
-                    const bool bad[3] = { b12, b13, b23 };
-                    const unsigned long long site =
-                        (unsigned long long)((long long)(z - 1) * N * (long long)N + (long long)roff);
-#pragma unroll
-                    for (int k = 0; k < 3; ++k)
-                        if (bad[k]) {
+                    for (int k = 0; k < 3; ++k) {
+                        if (cuts >> k & 1u) {
+                            const unsigned long long at =
+                                (unsigned long long)((long long)(z - 1) * N * (long long)N + (long long)roff);
                             const unsigned long long i = atomicAdd(da.list.count, 1ULL);
-                            if (i < (unsigned long long)da.list.capacity) da.list.items[i] = site * 4ULL + k;
+                            if (i < (unsigned long long)da.list.capacity) da.list.items[i] = at * 4ULL + k;
+                        } else {
+                            ic[k] += abs(q[k]);
+                            ic[3 + k] += q[k];
+                            ic[6] += q[k] != 0;
                         }
+                    }
                 }
             }
             if (z == z1) break;
             // energies and the Gauss residual of plane z
-            XiTerms xt;
             {
                 const real ti[3] = { t0[0], t0[0], t0[1] }, tij[3] = { t1y, nt[0], nt[1] };
                 const real tj[3] = { t0[1], t0[2], t0[2] }, tji[3] = { qx.d, qx.c, qy.c };
-                const real bsum = xi_terms(ti, tij, tj, tji, &xt);
+                unsigned wn;
+                const real bsum = xi_terms(ti, tij, tj, tji, &wn);
+                const unsigned wo = own_word(n, nc);
+                wm = ((wo + wn) & 0xffffffu) | ((wo | wn) & 0x07000000u);
                 real sn[3], co[3];
                 diag_links(t0, sn, co);
-                if (own) site(da, g_div, g_phi, f0, t0, sn, co, qx, qy, nf, bsum, mpr, mpi, m1, m2, m3, e1x, e2y, e3m);
+                if (own) site(sc, f0, t0, sn, co, qx, qy, nf, bsum, mpr, mpi, m1, m2, m3, e1x, e2y, e3m);
             }
-            xm = xt;
-            wm = w;
             e3m = m3;
             a0 = an;
         }
         __syncthreads();                         // the next column reuses the arrays
     }
 
-    __device__ __forceinline__ void site(const DiagArgs &da, DF g_div, DF g_phi, const real f0[2], const real t0[3],
+    __device__ __forceinline__ void site(const SiteCoef<real> &sc, const real f0[2], const real t0[3],
                                          const real sn[3], const real co[3], const D4<real> &qx, const D4<real> &qy,
                                          const real nf[2], real bsum, real pr, real pim, real e1, real e2, real e3,
                                          real e1b, real e2b, real e3b)
     {
-        const DiagCoef &dc = da.dc;
         const real fr[3] = { qx.a, qy.a, nf[0] }, fi[3] = { qx.b, qy.b, nf[1] };
         real g = real(0);
 #pragma unroll
@@ -359,11 +398,11 @@ struct DiagTile {
             g += a * a + b * b;
         }
         const real K = pr * pr + pim * pim;
-        const real G2 = g * (real)dc.inv_dx2;
-        const real m2 = f0[0] * f0[0] + f0[1] * f0[1] - (real)dc.sigma2;
-        const real V = (real)dc.v_coef * m2 * m2;
-        const real Eel = (real)dc.eel_coef * (e1 * e1 + e2 * e2 + e3 * e3);
-        const real B = (real)dc.b_coef * bsum;
+        const real G2 = g * sc.inv_dx2;
+        const real m2 = f0[0] * f0[0] + f0[1] * f0[1] - sc.sigma2;
+        const real V = sc.v_coef * m2 * m2;
+        const real Eel = sc.eel_coef * (e1 * e1 + e2 * e2 + e3 * e3);
+        const real B = sc.b_coef * bsum;
         const real L = K - G2 - V + Eel - B;
         const real rho = K + G2 + V + Eel + B;
         const real pp = K - G2 * real(1.0 / 3.0) - V + (Eel + B) * real(1.0 / 3.0);
@@ -373,19 +412,17 @@ struct DiagTile {
         ic[7] += !(isfinite(L) && isfinite(rho) && isfinite(pp));
         if constexpr (sizeof(real) == 8) {
             const double div = (e1 - e1b) + (e2 - e2b) + (e3 - e3b);
-            const double g1 = dc.g_div * div;
-            const double g2 = dc.g_phi * (f0[0] * pim - f0[1] * pr);
+            const double g1 = sc.g_div.h * div;
+            const double g2 = sc.g_phi.h * (f0[0] * pim - f0[1] * pr);
             const double Gs = g1 + g2, gs = fabs(g1) + fabs(g2);
             dg2 += Gs * Gs;
             dgs2 += gs * gs;
             dgmax = fmax(dgmax, fabs(Gs));
         } else {
-            const DF div = df_add(df_add(two_sum(e1, -e1b), two_sum(e2, -e2b)), two_sum(e3, -e3b));
-            const DF a = two_prod(f0[0], pim), b = two_prod(f0[1], pr);
-            const DF g1 = df_mul(g_div, div), g2 = df_mul(g_phi, df_add(a, { -b.h, -b.l }));
-            DF Gs = df_add(g1, g2);
+            const GaussTerms gt = gauss_terms(sc.g_div, sc.g_phi, f0[0], f0[1], pr, pim, e1, e1b, e2, e2b, e3, e3b);
+            DF Gs = gt.g;
             if (Gs.h < 0.f) Gs = { -Gs.h, -Gs.l };
-            const float gs = fabsf(g1.h) + fabsf(g2.h);
+            const float gs = gt.scale;
             const float sg = Gs.h * 0x1p30f, ss = gs * 0x1p30f;
             fg2.add(sg * sg);
             fgs2.add(ss * ss);

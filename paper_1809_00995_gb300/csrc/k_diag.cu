@@ -390,13 +390,13 @@ namespace {
 // taking every gridDim.x-th one; one partial per CTA.
 template <typename real, typename IT, int MINB>
 __global__ void __launch_bounds__(256, MINB)
-    k_diag_whole(View<real> v, int N, int tx, int ty, int items, int zc, DF g_div, DF g_phi, DiagArgs da)
+    k_diag_whole(View<real> v, int N, int tx, int ty, int items, int zc, SiteCoef<real> sc, DiagArgs da)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     DiagTile<real, IT> t;
     for (int it = blockIdx.x; it < items; it += gridDim.x) {
         const int bx = it % tx, by = (it / tx) % ty, z0 = it / (tx * ty) * zc;
-        t.column(v, N, da, g_div, g_phi, 32 * bx, 8 * by, z0, min(z0 + zc, N), smem_raw);
+        t.column(v, N, da, sc, 32 * bx, 8 * by, z0, min(z0 + zc, N), smem_raw);
     }
     t.flush(&da.partials[blockIdx.x]);
 }
@@ -432,8 +432,8 @@ cudaError_t launch_diag_whole_it(const View<real> &v, int N, const DiagArgs &da,
         configured |= dev_bit;
     }
     const DiagGrid g = diag_whole_grid<real>(N);
-    k_diag_whole<real, IT, minb><<<g.ctas, 256, smem, st>>>(v, N, g.tx, g.ty, g.items, g.zc, df_from(da.dc.g_div),
-                                                           df_from(da.dc.g_phi), da);
+    k_diag_whole<real, IT, minb><<<g.ctas, 256, smem, st>>>(v, N, g.tx, g.ty, g.items, g.zc, site_coef(da.dc, real(0)),
+                                                           da);
     return cudaGetLastError();
 }
 }  // namespace

@@ -118,13 +118,10 @@ struct Diag2Acc {
         s[7].add(K * L); s[8].add(G2 * L); s[9].add(pp * L); s[10].add(rho * L);
         tmax = fmaxf(tmax, fmaxf(fabsf(t1), fmaxf(fabsf(t2), fabsf(t3))));
         ic[7] += !(isfinite(L) && isfinite(rho) && isfinite(pp));
-        // Gauss residual in double-float arithmetic
-        const DF div = df_add(df_add(two_sum(e1, -e1b), two_sum(e2, -e2b)), two_sum(e3, -e3b));
-        const DF a = two_prod(f0.r, pim), b = two_prod(f0.i, pr);
-        const DF g1 = df_mul(c.g_div, div), gq = df_mul(c.g_phi, df_add(a, { -b.h, -b.l }));
-        DF Gs = df_add(g1, gq);
+        const GaussTerms gt = gauss_terms(c.g_div, c.g_phi, f0.r, f0.i, pr, pim, e1, e1b, e2, e2b, e3, e3b);
+        DF Gs = gt.g;
         if (Gs.h < 0.f) Gs = { -Gs.h, -Gs.l };
-        const float gs = fabsf(g1.h) + fabsf(gq.h);
+        const float gs = gt.scale;
         const float sg = Gs.h * 0x1p30f, ss = gs * 0x1p30f;
         g2.add(sg * sg);
         gs2.add(ss * ss);
