@@ -164,9 +164,49 @@ struct ah_sim {
     int64_t weak_launches;
     int diag_free_pairs;
     int64_t diag_step;
+    // device staging of field windows (FP64), kept between calls up to
+    // kScratchMax: allocating and freeing it takes longer than gathering and
+    // copying a small window (21 MB, a whole 64^3 state: 0.3 of 0.5 ms)
+    std::mutex scratch_mu;
+    double *scratch;
+    size_t scratch_bytes;
 };
 
 namespace {
+
+// Largest window staging buffer that a simulation keeps.
+constexpr size_t kScratchMax = (size_t)64 << 20;
+
+// Staging for one window of a call, held under the simulation's lock until the
+// call returns; windows above kScratchMax get a buffer of their own.
+struct Staging {
+    std::lock_guard<std::mutex> lk;
+    double *p = nullptr;
+    bool own = false;
+    cudaError_t err = cudaSuccess;
+    Staging(ah_sim *h, size_t bytes) : lk(h->scratch_mu)
+    {
+        if (bytes > kScratchMax) {
+            own = true;
+            err = cudaMalloc(&p, bytes);
+            if (err != cudaSuccess) p = nullptr;
+            return;
+        }
+        if (bytes > h->scratch_bytes) {
+            // no work uses the old buffer: every call waits for its copies
+            cudaFree(h->scratch);
+            h->scratch = nullptr;
+            h->scratch_bytes = 0;
+            err = cudaMalloc(&h->scratch, bytes);
+            if (err != cudaSuccess) { h->scratch = nullptr; return; }
+            h->scratch_bytes = bytes;
+        }
+        p = h->scratch;
+    }
+    ~Staging() { if (own) cudaFree(p); }
+    Staging(const Staging &) = delete;
+    Staging &operator=(const Staging &) = delete;
+};
 
 // Largest fraction of pierced plaquettes at which a deferred observables pass
 // rides on the next two-step launch (k_fused2_diag) without AH_FLAG_FUSED_DIAG.
@@ -443,11 +483,7 @@ ah_status do_diag(ah_sim *h, Box b, ah_obs *out)
     else
         AH_CUDA(launch_diag<real>(v, h->N, b, dc, h->partials, h->diag_blocks, h->result, h->list, exact,
                                   h->stream));
-    AH_CUDA(cudaMemcpyAsync(h->host_result, h->result, sizeof(DiagPartial), cudaMemcpyDeviceToHost,
-                            h->stream));
-    AH_CUDA(cudaMemcpyAsync(h->host_count, h->list.count, sizeof(unsigned long long),
-                            cudaMemcpyDeviceToHost, h->stream));
-    AH_CUDA(cudaMemcpyAsync(h->host_err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    AH_CUDA(cudaMemcpyAsync(h->host_result, h->result, sizeof(DiagPartial) + 16, cudaMemcpyDeviceToHost, h->stream));
     AH_CUDA(cudaStreamSynchronize(h->stream));
     if (*h->host_err) return check_device_error(h);
     if (!exact && *h->host_count > (unsigned long long)h->list.capacity) {
@@ -646,9 +682,10 @@ ah_status ah_create_ex(const ah_config *cfg, ah_sim **out)
     // expected near-cut plaquettes: about 5e-5 of the 3 N^3 plaquettes in FP32
     h->list.capacity = std::max<long long>(1LL << 20, h->nsites * 3 / 2000);
     e = cudaMalloc(&h->dmem, h->dbytes);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&h->partials, sizeof(DiagPartial) * (nparts + 1));
-    if (e == cudaSuccess)
-        e = cudaMalloc((void **)&h->list.count, sizeof(unsigned long long) * (1 + h->list.capacity));
+    // the partials, then what a pass reports in one copy: the sums, the count of
+    // listed plaquettes and the error word of the bounded waits
+    if (e == cudaSuccess) e = cudaMalloc((void **)&h->partials, sizeof(DiagPartial) * (nparts + 1) + 16);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&h->list.items, sizeof(unsigned long long) * h->list.capacity);
     if (e == cudaSuccess) e = cudaMallocHost((void **)&h->host_result, sizeof(DiagPartial) + 32);
     if (e != cudaSuccess) {
         const double gb = h->dbytes / 1e9;
@@ -657,14 +694,14 @@ ah_status ah_create_ex(const ah_config *cfg, ah_sim **out)
         return fail(AH_ERR_OOM, "allocation of %.3g GB failed: %s", gb, cudaGetErrorString(e));
     }
     h->result = h->partials + nparts;
-    h->list.items = h->list.count + 1;
+    h->list.count = (unsigned long long *)(h->result + 1);
+    h->d_err = (int *)(h->list.count + 1);
     h->host_count = (unsigned long long *)(h->host_result + 1);
     h->host_err = (int *)(h->host_count + 1);
-    e = cudaMalloc((void **)&h->d_err, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->d_err, 0, sizeof(int), h->stream);
+    e = cudaMemsetAsync(h->d_err, 0, sizeof(int), h->stream);
     if (e != cudaSuccess) {
         ah_destroy(h);
-        return fail(AH_ERR_OOM, "allocation failed: %s", cudaGetErrorString(e));
+        return fail(AH_ERR_CUDA, "initialisation failed: %s", cudaGetErrorString(e));
     }
     if (cfg->precision == AH_FP32) carve(h->f32, (char *)h->dmem, (size_t)h->nsites, h->two_step);
     else carve(h->f64, (char *)h->dmem, (size_t)h->nsites);
@@ -837,14 +874,14 @@ ah_status ah_get_fields(ah_sim *h, int32_t x0, int32_t y0, int32_t z0, int32_t n
     auto md = [N](int v) { v %= N; return v < 0 ? v + N : v; };
     const Box b{ md(x0), md(y0), md(z0), nx, ny, nz };
     const size_t bytes = sizeof(double) * 10 * (size_t)nx * ny * nz;
-    double *tmp = nullptr;
-    AH_CUDA(cudaMalloc(&tmp, bytes));
+    const Staging buf(h, bytes);
+    AH_CUDA(buf.err);
+    double *const tmp = buf.p;
     cudaError_t e = h->cfg.precision == AH_FP32
                         ? launch_gather_window<float>(h->f32, h->cur, N, b, tmp, h->stream)
                         : launch_gather_window<double>(h->f64, h->cur, N, b, tmp, h->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(out, tmp, bytes, cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    cudaFree(tmp);
     if (e != cudaSuccess) return fail(AH_ERR_CUDA, "get_fields failed: %s", cudaGetErrorString(e));
     return AH_OK;
 }
@@ -856,14 +893,14 @@ ah_status ah_set_fields(ah_sim *h, const double *in, int64_t step)
     if (!in || step < 0) return fail(AH_ERR_ARG, "null input or negative step");
     if ((st = diag_fence(h)) != AH_OK) return st;
     const size_t bytes = sizeof(double) * 10 * (size_t)h->nsites;
-    double *tmp = nullptr;
-    AH_CUDA(cudaMalloc(&tmp, bytes));
+    const Staging buf(h, bytes);
+    AH_CUDA(buf.err);
+    double *const tmp = buf.p;
     cudaError_t e = cudaMemcpyAsync(tmp, in, bytes, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess)
         e = h->cfg.precision == AH_FP32 ? launch_scatter_all<float>(h->f32, h->cur, h->N, tmp, h->stream)
                                         : launch_scatter_all<double>(h->f64, h->cur, h->N, tmp, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    cudaFree(tmp);
     if (e != cudaSuccess) return fail(AH_ERR_CUDA, "set_fields failed: %s", cudaGetErrorString(e));
     h->step = step;
     h->pristine = false;
@@ -1002,8 +1039,8 @@ void ah_destroy(ah_sim *h)
     if (h->ev_done) cudaEventDestroy(h->ev_done);
     if (h->dmem) cudaFree(h->dmem);
     if (h->partials) cudaFree(h->partials);
-    if (h->list.count) cudaFree(h->list.count);
-    if (h->d_err) cudaFree(h->d_err);
+    if (h->list.items) cudaFree(h->list.items);
+    cudaFree(h->scratch);
     if (h->host_result) cudaFreeHost(h->host_result);
     if (h->stream && h->own_stream) cudaStreamDestroy(h->stream);
     delete h;
