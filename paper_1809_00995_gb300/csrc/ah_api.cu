@@ -651,7 +651,7 @@ ah_status ah_create_ex(const ah_config *cfg, ah_sim **out)
     h->cfg = *cfg;
     if (h->cfg.kernel == AH_KERNEL_AUTO) h->cfg.kernel = AH_KERNEL_FUSED;
     h->N = cfg->N;
-    h->variant = cfg->precision == AH_FP32 ? fused_default_variant<float>() : fused_default_variant<double>();
+    h->variant = cfg->precision == AH_FP32 ? fused_default_variant<float>(cfg->N) : fused_default_variant<double>(cfg->N);
     h->two_step = (cfg->flags & AH_FLAG_TWO_STEP) != 0;
     h->variant2 = fused2_default_variant();
     // fault injection for tests, read at creation: AH_TMA_DROP_COPY=q makes the

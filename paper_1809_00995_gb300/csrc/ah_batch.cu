@@ -40,7 +40,7 @@ using namespace ah;
 
 namespace {
 
-constexpr int kZChunk = 64;        // planes per work item
+constexpr int kZChunk = 64;        // most planes per work item
 constexpr int kZChunk2 = 256;      // planes per two-step work item (each also runs two extra planes)
 // Two-step batches step the lattices of at least this side in pairs and the
 // smaller ones one step per launch: the two-step tile writes 30 x 6 of its
@@ -176,11 +176,12 @@ struct Engine {
     int shape2 = 0;                    // shape of the batched two-step pass
     BatchLattice *d_lat = nullptr;
     BatchState *d_state = nullptr;
-    int2 *d_items = nullptr, *d_items2 = nullptr;
-    int *d_nitems = nullptr;           // [0] single-step items, [1] two-step items
+    // work items: single step (kernel of `shape`, then that of feed_lattice), two-step pass
+    int2 *d_items = nullptr, *d_itemsf = nullptr, *d_items2 = nullptr;
+    int *d_nitems = nullptr;           // their numbers: [0], [2], [1]
     unsigned int *d_counter = nullptr;
     int cap_lat = 0;
-    long long cap_items = 0, cap_items2 = 0;
+    long long cap_items = 0, cap_itemsf = 0, cap_items2 = 0;
     DiagPartial *d_partials = nullptr, *d_result = nullptr, *h_result = nullptr;
     int nparts = 0;                    // entries of d_partials before d_result
     DiagList list{};
@@ -207,9 +208,9 @@ struct Engine {
         if (e == cudaSuccess) e = cudaMalloc(&d_partials, sizeof(DiagPartial) * (nparts + 1));
         if (e == cudaSuccess) e = cudaMalloc(&list.count, sizeof(unsigned long long) * (1 + list.capacity));
         if (e == cudaSuccess) e = cudaMallocHost(&h_result, sizeof(DiagPartial) + 64);
-        if (e == cudaSuccess) e = cudaMalloc(&d_nitems, 2 * sizeof(int));
-        if (e == cudaSuccess) e = cudaMalloc(&d_counter, sizeof(unsigned int));
-        if (e == cudaSuccess) e = cudaMemsetAsync(d_counter, 0, sizeof(unsigned int), st);
+        if (e == cudaSuccess) e = cudaMalloc(&d_nitems, 3 * sizeof(int));
+        if (e == cudaSuccess) e = cudaMalloc(&d_counter, 2 * sizeof(unsigned int));
+        if (e == cudaSuccess) e = cudaMemsetAsync(d_counter, 0, 2 * sizeof(unsigned int), st);
         if (e != cudaSuccess) return e;
         d_result = d_partials + nparts;
         list.items = list.count + 1;
@@ -227,12 +228,39 @@ struct Engine {
     {
         if (st) cudaStreamSynchronize(st);
         clear_graphs();
-        cudaFree(d_lat); cudaFree(d_state); cudaFree(d_items); cudaFree(d_items2);
+        cudaFree(d_lat); cudaFree(d_state); cudaFree(d_items); cudaFree(d_itemsf); cudaFree(d_items2);
         cudaFree(d_nitems); cudaFree(d_counter); cudaFree(d_partials);
         if (list.count) cudaFree(list.count);
         if (h_result) cudaFreeHost(h_result);
         if (st) cudaStreamDestroy(st);
         *this = Engine();
+    }
+
+    // Planes per work item of the single step of the lattices with feed_lattice(N)
+    // == feed: their items share the resident CTAs, so a launch takes about (all
+    // items' planes, two more per item) / slots and ends unevenly by half an item;
+    // the chunk that makes that least.  (A lone 64^3 lattice is 8 items of 64 planes
+    // or 128 of 4.)
+    int item_planes(const std::vector<Lat *> &lats, bool feed) const
+    {
+        const long long slots = (long long)num_sms * batch_resident_ctas(shape, feed);
+        int best = kZChunk;
+        long long best_cost = -1;
+        for (int zc = kZChunk; zc >= 2; zc /= 2) {
+            long long planes = 0;
+            for (const Lat *L : lats) {
+                if (feed_lattice(L->N) != feed) continue;
+                int tx, ty;
+                batch_tiles(shape, L->N, &tx, &ty);
+                planes += (long long)tx * ty * (L->N + 2 * ((L->N + zc - 1) / zc));
+            }
+            const long long cost = 2 * planes + slots * zc;
+            if (best_cost < 0 || cost < best_cost) {
+                best_cost = cost;
+                best = zc;
+            }
+        }
+        return best;
     }
 
     // Upload descriptors, states and work items of the lattices (largest first).
@@ -241,9 +269,10 @@ struct Engine {
         const int n = (int)lats.size();
         std::vector<BatchLattice> bl(n);
         std::vector<BatchState> bs(n);
-        std::vector<int2> items, items2;
+        std::vector<int2> items, itemsf, items2;
         std::vector<int> order(n);
         for (int i = 0; i < n; ++i) order[i] = i;
+        const int zchunk[2] = { item_planes(lats, false), item_planes(lats, true) };
         std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return lats[a]->N > lats[b]->N; });
         for (int i = 0; i < n; ++i) {
             const Lat &L = *lats[i];
@@ -257,7 +286,7 @@ struct Engine {
             }
             B.N = L.N;
             batch_tiles(shape, L.N, &B.tiles_x, &B.tiles_y);
-            B.zc = std::min(L.N, kZChunk);
+            B.zc = std::min(L.N, zchunk[feed_lattice(L.N)]);
             B.nchunk = (L.N + B.zc - 1) / B.zc;
             if (two && L.two) {
                 B.pairs = 1;
@@ -275,7 +304,8 @@ struct Engine {
         direct.clear();
         for (int i : order) {
             const int cnt = bl[i].tiles_x * bl[i].tiles_y * bl[i].nchunk;
-            for (int k = 0; k < cnt; ++k) items.push_back(make_int2(i, k));
+            auto &list = feed_lattice(lats[i]->N) ? itemsf : items;
+            for (int k = 0; k < cnt; ++k) list.push_back(make_int2(i, k));
             if (bl[i].pairs && lats[i]->N >= kDirectMinN) {
                 direct.push_back(lats[i]);           // its own grid launches, no items
                 continue;
@@ -303,20 +333,32 @@ struct Engine {
             e = cudaMalloc(&d_items2, sizeof(int2) * cap_items2);
             clear_graphs();
         }
-        const int ni[2] = { (int)items.size(), (int)items2.size() };
+        if (e == cudaSuccess && (long long)itemsf.size() > cap_itemsf) {
+            cudaFree(d_itemsf);
+            cap_itemsf = std::max<long long>((long long)itemsf.size(), 2 * cap_itemsf);
+            e = cudaMalloc(&d_itemsf, sizeof(int2) * cap_itemsf);
+            clear_graphs();
+        }
+        const int ni[3] = { (int)items.size(), (int)items2.size(), (int)itemsf.size() };
         if (e == cudaSuccess && n) e = cudaMemcpyAsync(d_lat, bl.data(), sizeof(BatchLattice) * n, cudaMemcpyHostToDevice, st);
         if (e == cudaSuccess && n) e = cudaMemcpyAsync(d_state, bs.data(), sizeof(BatchState) * n, cudaMemcpyHostToDevice, st);
         if (e == cudaSuccess && ni[0])
             e = cudaMemcpyAsync(d_items, items.data(), sizeof(int2) * ni[0], cudaMemcpyHostToDevice, st);
         if (e == cudaSuccess && ni[1])
             e = cudaMemcpyAsync(d_items2, items2.data(), sizeof(int2) * ni[1], cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(d_nitems, ni, 2 * sizeof(int), cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess && ni[2])
+            e = cudaMemcpyAsync(d_itemsf, itemsf.data(), sizeof(int2) * ni[2], cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(d_nitems, ni, 3 * sizeof(int), cudaMemcpyHostToDevice, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // host vectors above
         nlat_loaded = n;
+        plain = { d_items, d_nitems, ni[0] > 0 };
+        feed = { d_itemsf, d_nitems + 2, ni[2] > 0 };
         n_paired = n_unpaired = 0;
         for (int i = 0; i < n; ++i) (bl[i].pairs ? n_paired : n_unpaired) += 1;
         return e;
     }
+    BatchItems plain{}, feed{};
+    int single_launches() const { return plain.any + feed.any + 1; }   // kernels of one single step
     int n_paired = 0, n_unpaired = 0;   // loaded lattices stepped in pairs / one step at a time
     std::vector<Lat *> direct;          // paired lattices run by the single-lattice two-step kernel
 
@@ -354,9 +396,8 @@ struct Engine {
     {
         if (two) {
             auto single = [&](int mode) {
-                launches += 2;
-                return launch_fused_batch(shape, d_lat, d_state, nlat_loaded, d_items, d_nitems, d_counter, num_sms, st,
-                                          mode);
+                launches += single_launches();
+                return launch_fused_batch(shape, d_lat, d_state, nlat_loaded, plain, feed, d_counter, num_sms, st, mode);
             };
             for (int r = 0; r < R / 2; ++r) {
                 for (const Lat *L : direct) {
@@ -384,10 +425,9 @@ struct Engine {
             return cudaSuccess;
         }
         for (int r = 0; r < R; ++r) {
-            cudaError_t e = launch_fused_batch(shape, d_lat, d_state, nlat_loaded, d_items, d_nitems, d_counter,
-                                               num_sms, st);
+            cudaError_t e = launch_fused_batch(shape, d_lat, d_state, nlat_loaded, plain, feed, d_counter, num_sms, st);
             if (e != cudaSuccess) return e;
-            launches += 2;
+            launches += single_launches();
         }
         return cudaSuccess;
     }
@@ -403,8 +443,8 @@ struct Engine {
         // kernel parameters, which change from round to round: no graph then
         if (!use_graph || !direct.empty()) return enqueue_steps(R);
         const long long before = launches;
-        const int mix = (n_paired ? 1 : 0) + (n_unpaired ? 2 : 0);
-        const auto key = std::make_tuple(two ? 1000 + 64 * mix + 16 * shape2 + shape : shape, R, nlat_loaded);
+        const int mix = (n_paired ? 1 : 0) + (n_unpaired ? 2 : 0) + (plain.any ? 4 : 0) + (feed.any ? 8 : 0);
+        const auto key = std::make_tuple((two ? 1024 : 0) + 64 * mix + 16 * shape2 + shape, R, nlat_loaded);
         auto it = graphs.find(key);
         if (it == graphs.end()) {
             cudaGraph_t g;
@@ -420,8 +460,9 @@ struct Engine {
             it = graphs.emplace(key, ex).first;
             launches = before;
         }
-        launches = before + (two ? 2LL * ((R / 2) * ((n_paired ? 1 : 0) + (n_unpaired ? 2 : 0)) + R % 2)
-                                 : 2LL * R);
+        const long long single = single_launches();
+        launches = before + (two ? (R / 2) * (n_paired ? 2LL : 0LL) + ((R / 2) * (n_unpaired ? 2 : 0) + R % 2) * single
+                                 : single * R);
         return cudaGraphLaunch(it->second, st);
     }
 

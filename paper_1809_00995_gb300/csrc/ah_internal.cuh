@@ -146,7 +146,7 @@ const char *fused_variant_name(int variant);
 template <typename real>
 bool fused_variant_ok(int variant, int N);
 template <typename real>
-int fused_default_variant();
+int fused_default_variant(int N);
 
 // Two leapfrog steps (coefficients c1 for step n, c2 for step n + 1) in one
 // pass, FP32; shape `variant` in [0, fused2_variant_count()).
@@ -268,14 +268,26 @@ __host__ __device__ inline bool batch_takes_single(const BatchLattice &B, int n,
 int batch_shape_count();
 bool batch_shape_ok(int shape, int N);
 void batch_tiles(int shape, int N, int *tx, int *ty);
+int batch_resident_ctas(int shape, bool feed);      // per SM, as the registers allow
 // Per-shape one-time set-up (kernel attributes, occupancy) of the batched
 // single-step kernel, or of the batched two-step pass if `two`, outside any
 // stream capture.
 cudaError_t batch_shape_prepare(int shape, int num_sms, cudaStream_t st, bool two = false);
-// mode: which lattices take part (BATCH_ALL, BATCH_UNPAIRED, BATCH_ROUND_END).
-cudaError_t launch_fused_batch(int shape, const BatchLattice *lat, BatchState *state, int nlat, const int2 *items,
-                               const int *nitems, unsigned int *counter, int num_sms, cudaStream_t st,
-                               int mode = BATCH_ALL);
+// Work items of one of the two single-step kernels: device list and count, and
+// whether there are any (else the kernel is not launched).
+struct BatchItems {
+    const int2 *items;
+    const int *count;
+    bool any;
+};
+// Lattices whose single steps run the kernel that ah_step runs for them by
+// default (feed_tile.cuh), in their own item list; the others run `shape`.
+bool feed_lattice(int N);
+// mode: which lattices take part (BATCH_ALL, BATCH_UNPAIRED, BATCH_ROUND_END);
+// counter: two work counters.
+cudaError_t launch_fused_batch(int shape, const BatchLattice *lat, BatchState *state, int nlat,
+                               const BatchItems &plain, const BatchItems &feed, unsigned int *counter, int num_sms,
+                               cudaStream_t st, int mode = BATCH_ALL);
 // Batched two-step pass (two leapfrog steps of every lattice per launch),
 // shapes 0 (32 x 8 CTA tile, 3 CTAs per SM) and 1 (32 x 12, 2 per SM).
 int batch2_shape_count();

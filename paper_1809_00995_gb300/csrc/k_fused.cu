@@ -28,6 +28,7 @@
 #include "ah_internal.cuh"
 #include "sincos32.cuh"
 #include "fused_common.cuh"
+#include "feed_tile.cuh"
 #include "step_tile.cuh"
 
 namespace ah {
@@ -293,6 +294,14 @@ __global__ void __launch_bounds__(256, MINB) k_fused(View<real> v, int N, int zc
         fused_tile<real, TY, RX, IT>(v, N, zc, c, blockIdx.x, blockIdx.y, blockIdx.z, smem_raw);
 }
 
+// The step of two rows per thread with copied planes (feed_tile.cuh).
+template <int NP, int MINB, typename IT>
+__global__ void __launch_bounds__(32 * NP, MINB) k_feed(View<float> v, int N, int zc, KickCoef2 c)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    feed_tile<NP, IT>(v, N, zc, c, blockIdx.x, blockIdx.y, blockIdx.z, smem_raw);
+}
+
 // Batched fused step: persistent CTAs take (lattice, tile) work items from a
 // shared counter and advance every lattice of the batch by one step.  Lattices
 // that have run all their steps are skipped; each lattice's step number, read
@@ -331,8 +340,49 @@ k_fused_batch(const BatchLattice *lat, BatchState *state, const int2 *items, con
     }
 }
 
+// The same for the lattices that ah_step steps with k_feed (feed_lattice).  The
+// item's pointers and coefficients are in shared memory, where they cost no
+// registers.
+template <int NP, int MINB>
+__global__ void __launch_bounds__(32 * NP, MINB)
+    k_feed_batch(const BatchLattice *lat, BatchState *state, const int2 *items, const int *nitems,
+                 unsigned int *counter, int mode)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int s_item;
+    __shared__ View<float> sv;
+    __shared__ KickCoef2 sc;
+    const int n = *nitems;
+    for (;;) {
+        if (threadIdx.x == 0) s_item = (int)atomicAdd(counter, 1u);
+        __syncthreads();
+        const int it = s_item;
+        if (it >= n) break;
+        const int L = items[it].x, local = items[it].y;
+        const BatchLattice &B = lat[L];
+        const int step = state[L].step;
+        const bool takes = batch_takes_single(B, step, mode);
+        if (takes && threadIdx.x == 0) {
+            const int cur = state[L].cur, o = 1 - cur;
+            float *const *q = B.q[state[L].pe];
+            sv.phr = B.F.phr[cur]; sv.phi = B.F.phi[cur];
+            sv.th1 = B.F.th[cur][0]; sv.th2 = B.F.th[cur][1]; sv.th3 = B.F.th[cur][2];
+            sv.pir = q[0]; sv.pii = q[1]; sv.e1 = q[2]; sv.e2 = q[3]; sv.e3 = q[4];
+            sv.ophr = B.F.phr[o]; sv.ophi = B.F.phi[o];
+            sv.oth1 = B.F.th[o][0]; sv.oth2 = B.F.th[o][1]; sv.oth3 = B.F.th[o][2];
+            sc = pair_coef(B.coefs[step]);
+        }
+        __syncthreads();
+        if (takes) {
+            const int bx = local % B.tiles_x, by = (local / B.tiles_x) % B.tiles_y;
+            feed_tile<NP, int>(sv, B.N, B.zc, sc, bx, by, local / (B.tiles_x * B.tiles_y), smem_raw);
+        }
+        __syncthreads();
+    }
+}
+
 // After a batched step: every lattice that took part (batch_takes_single)
-// moves to its next step and swaps its phi/theta buffers; the work counter is
+// moves to its next step and swaps its phi/theta buffers; the work counters are
 // reset.
 __global__ void k_batch_advance(const BatchLattice *lat, BatchState *state, int nlat, unsigned int *counter,
                                 int mode)
@@ -343,7 +393,7 @@ __global__ void k_batch_advance(const BatchLattice *lat, BatchState *state, int 
             state[L].cur ^= 1;
         }
     }
-    if (threadIdx.x == 0) *counter = 0u;
+    if (threadIdx.x < 2) counter[threadIdx.x] = 0u;
 }
 
 // Compile-time shapes of the fused step: tile height TY (TY/8 rows per thread),
@@ -404,6 +454,37 @@ constexpr PlaneTimes kStepTimes32 = { { 113, 156, 199, 255 } };
 // FP64 step: bound by the FP64 pipe, which one CTA fills to 0.88
 constexpr PlaneTimes kStepTimes64 = { { 123, 216, 324, 432 } };
 
+// z chunks of the k_feed grid: at most 64 planes, since CTAs of longer marches
+// drift apart until the rows they share no longer meet in L2 (1024^3: 4 chunks read
+// 62 B per site and take 17.3 ms, 16 chunks 13.8).
+constexpr PlaneTimes kFeedTimes = { { 140, 214 } };
+constexpr int kFeedMaxChunk = 64;
+
+template <typename IT>
+cudaError_t launch_feed_it(const View<float> &v, int N, const KickCoef<float> &c, cudaStream_t st)
+{
+    constexpr int NP = 8, MINB = 2;
+    using G = FeedGeo<NP>;
+    static unsigned long long configured = 0;   // per device, once per instantiation
+    const unsigned long long dev_bit = 1ULL << device_slot();
+    if (!(configured & dev_bit)) {
+        const cudaError_t e = cudaFuncSetAttribute(k_feed<NP, MINB, IT>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::smem);
+        if (e != cudaSuccess) return e;
+        configured |= dev_bit;
+    }
+    const int tx = (N + 31) / 32, ty = (N + G::TY - 1) / G::TY;
+    const int n = std::max(choose_chunks(N, (long long)tx * ty, MINB, 2, kFeedTimes),
+                           (N + kFeedMaxChunk - 1) / kFeedMaxChunk);
+    const int zc = (N + n - 1) / n;
+    k_feed<NP, MINB, IT><<<dim3(tx, ty, (N + zc - 1) / zc), G::NT, G::smem, st>>>(v, N, zc, pair_coef(c));
+    return cudaGetLastError();
+}
+cudaError_t launch_feed(const View<float> &v, int N, const KickCoef<float> &c, cudaStream_t st)
+{
+    return (long long)N * N * N < (1LL << 31) ? launch_feed_it<int>(v, N, c, st) : launch_feed_it<long long>(v, N, c, st);
+}
+
 template <typename real, int TY, int RX, int MINB>
 cudaError_t launch_shape(const View<real> &v, int N, const KickCoef<real> &c, int min_chunk, bool wave_model,
                          cudaStream_t st)
@@ -441,12 +522,14 @@ cudaError_t launch_shape(const View<real> &v, int N, const KickCoef<real> &c, in
 
 }  // namespace
 
-// Shape used when a simulation is not autotuned: the fastest on GB300 at
-// 512^3 and 1024^3 (any N; RX = 1).
+// Shape used when a simulation is not autotuned.  FP32: from 64^3 on, where rows can
+// be copied in 16 bytes, ty16_b2_w (feed_tile.cuh; it ties at 64^3, 10.3 us, and wins
+// from 96^3 on, 18.5 against 20.6 us), else ty8_b4_w, the fastest of the others at
+// every measured size from 24^3 to 1024^3.
 template <>
-int fused_default_variant<float>() { return 10; }      // ty8_b4_w
+int fused_default_variant<float>(int N) { return feed_ok(N) && N >= 64 ? 13 : 10; }
 template <>
-int fused_default_variant<double>() { return 3; }      // ty8_b2_w
+int fused_default_variant<double>(int) { return 3; }      // ty8_b2_w
 
 template <>
 int fused_variant_count<float>() { return (int)(sizeof(kVariants32) / sizeof(kVariants32[0])); }
@@ -469,6 +552,9 @@ cudaError_t launch_fused_step<float>(const View<float> &v, int N, const KickCoef
     if (variant < 0 || variant >= fused_variant_count<float>()) return cudaErrorInvalidValue;
     const int mc = kVariants32[variant].min_chunk;
     const bool wm = kVariants32[variant].wave_model;
+    // ty16_b2_w: two rows per thread; where rows can be copied in 16 bytes, from
+    // copied planes
+    if (variant == 13 && feed_ok(N)) return launch_feed(v, N, c, st);
     switch (variant) {
     case 0: return launch_shape<float, 16, 1, 2>(v, N, c, mc, wm, st);
     case 1: return launch_shape<float, 16, 1, 3>(v, N, c, mc, wm, st);
@@ -510,8 +596,8 @@ struct BatchShape { int ty, rx, minb; };
 constexpr BatchShape kBatchShapes[] = { { 8, 1, 4 }, { 16, 1, 2 }, { 8, 2, 2 } };
 
 template <int TY, int RX, int MINB>
-cudaError_t launch_batch_shape(const BatchLattice *lat, BatchState *state, int nlat, const int2 *items,
-                               const int *nitems, unsigned int *counter, int num_sms, cudaStream_t st, int mode)
+cudaError_t launch_batch_shape(const BatchLattice *lat, BatchState *state, const int2 *items, const int *nitems,
+                               unsigned int *counter, int num_sms, cudaStream_t st, int mode)
 {
     using G = Geo<float, TY, RX>;
     static int blocks_per_sm_dev[64] = {};      // per device
@@ -527,7 +613,22 @@ cudaError_t launch_batch_shape(const BatchLattice *lat, BatchState *state, int n
     }
     k_fused_batch<TY, RX, MINB><<<num_sms * blocks_per_sm, 256, G::smem, st>>>(lat, state, items, nitems, counter,
                                                                               mode);
-    k_batch_advance<<<1, 256, 0, st>>>(lat, state, nlat, counter, mode);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_feed_batch(const BatchLattice *lat, BatchState *state, const int2 *items, const int *nitems,
+                              unsigned int *counter, int num_sms, cudaStream_t st, int mode)
+{
+    using G = FeedGeo<8>;
+    static unsigned long long configured = 0;   // per device
+    const unsigned long long dev_bit = 1ULL << device_slot();
+    if (!(configured & dev_bit)) {
+        const cudaError_t e = cudaFuncSetAttribute(k_feed_batch<8, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)G::smem);
+        if (e != cudaSuccess) return e;
+        configured |= dev_bit;
+    }
+    k_feed_batch<8, 2><<<num_sms * 2, G::NT, G::smem, st>>>(lat, state, items, nitems, counter, mode);
     return cudaGetLastError();
 }
 }  // namespace
@@ -552,9 +653,9 @@ cudaError_t batch_shape_prepare(int shape, int num_sms, cudaStream_t st, bool tw
         unsigned int *c = nullptr;
         cudaError_t e = cudaMalloc(&a, sizeof(BatchState));
         if (e == cudaSuccess) e = cudaMalloc(&z, sizeof(int));
-        if (e == cudaSuccess) e = cudaMalloc(&c, sizeof(unsigned int));
+        if (e == cudaSuccess) e = cudaMalloc(&c, 2 * sizeof(unsigned int));
         if (e == cudaSuccess) e = cudaMemsetAsync(z, 0, sizeof(int), st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(c, 0, sizeof(unsigned int), st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c, 0, 2 * sizeof(unsigned int), st);
         if (e != cudaSuccess) {
             cudaFree(a); cudaFree(z); cudaFree(c);
             return e;
@@ -563,28 +664,46 @@ cudaError_t batch_shape_prepare(int shape, int num_sms, cudaStream_t st, bool tw
     }
     // nlat = 0: the advance kernel touches no lattice; nitems = 0: no work
     if (two) return launch_fused2_batch(shape, nullptr, d_dummy, 0, nullptr, d_zero, d_cnt, num_sms, st);
-    return launch_fused_batch(shape, nullptr, d_dummy, 0, nullptr, d_zero, d_cnt, num_sms, st);
+    const BatchItems none = { nullptr, d_zero, true };
+    return launch_fused_batch(shape, nullptr, d_dummy, 0, none, none, d_cnt, num_sms, st);
 }
+
+bool feed_lattice(int N) { return fused_default_variant<float>(N) == 13; }
 
 void batch_tiles(int shape, int N, int *tx, int *ty)
 {
+    if (feed_lattice(N)) {
+        *tx = (N + 31) / 32;
+        *ty = (N + FeedGeo<8>::TY - 1) / FeedGeo<8>::TY;
+        return;
+    }
     const BatchShape &b = kBatchShapes[shape];
     *tx = (N + 32 * b.rx - 1) / (32 * b.rx);
     *ty = (N + b.ty - 1) / b.ty;
 }
 
+int batch_resident_ctas(int shape, bool feed) { return feed ? 2 : kBatchShapes[shape].minb; }
+
 bool batch_shape_ok(int shape, int N) { return kBatchShapes[shape].rx == 1 || N % 2 == 0; }
 
-cudaError_t launch_fused_batch(int shape, const BatchLattice *lat, BatchState *state, int nlat, const int2 *items,
-                               const int *nitems, unsigned int *counter, int num_sms, cudaStream_t st,
-                               int mode)
+cudaError_t launch_fused_batch(int shape, const BatchLattice *lat, BatchState *state, int nlat,
+                               const BatchItems &plain, const BatchItems &feed, unsigned int *counter, int num_sms,
+                               cudaStream_t st, int mode)
 {
-    switch (shape) {
-    case 0: return launch_batch_shape<8, 1, 4>(lat, state, nlat, items, nitems, counter, num_sms, st, mode);
-    case 1: return launch_batch_shape<16, 1, 2>(lat, state, nlat, items, nitems, counter, num_sms, st, mode);
-    case 2: return launch_batch_shape<8, 2, 2>(lat, state, nlat, items, nitems, counter, num_sms, st, mode);
-    default: return cudaErrorInvalidValue;
+    cudaError_t e = cudaSuccess;
+    if (plain.any) {
+        switch (shape) {
+        case 0: e = launch_batch_shape<8, 1, 4>(lat, state, plain.items, plain.count, counter, num_sms, st, mode); break;
+        case 1: e = launch_batch_shape<16, 1, 2>(lat, state, plain.items, plain.count, counter, num_sms, st, mode); break;
+        case 2: e = launch_batch_shape<8, 2, 2>(lat, state, plain.items, plain.count, counter, num_sms, st, mode); break;
+        default: e = cudaErrorInvalidValue;
+        }
     }
+    if (e == cudaSuccess && feed.any)
+        e = launch_feed_batch(lat, state, feed.items, feed.count, counter + 1, num_sms, st, mode);
+    if (e != cudaSuccess) return e;
+    k_batch_advance<<<1, 256, 0, st>>>(lat, state, nlat, counter, mode);
+    return cudaGetLastError();
 }
 
 }  // namespace ah
