@@ -178,19 +178,17 @@ template <typename real>
 cudaError_t launch_wind_recount_on_overflow(const View<real> &v, int N, DiagList list, DiagPartial *result,
                                             int nblocks, cudaStream_t st);
 
-// Whole-lattice diagnostics on a z-marching tile walk (diag_tile.cuh): one
-// DiagPartial per persistent CTA (at most fused_diag_max_ctas of them,
-// whatever N), near-cut
-// plaquettes appended to the list.
+// Whole-lattice diagnostics on a z-marching tile walk (diag_tile.cuh,
+// diag_pair.cuh): one DiagPartial per persistent CTA (at most
+// fused_diag_max_ctas of them, whatever N), near-cut plaquettes appended to the
+// list.
 struct DiagArgs {
     DiagCoef dc;
     DiagPartial *partials;
     DiagList list;
 };
 int fused_diag_max_ctas();
-template <typename real>
-cudaError_t launch_fused_diag(const View<real> &v, int N, const DiagArgs &da, cudaStream_t st);
-// The whole fast diagnostic: clear the list, launch_fused_diag, sum the
+// The whole fast diagnostic: clear the list, the tile walk, sum the
 // partials in a fixed order into *result, FP64 windings of the listed
 // plaquettes (fix_blocks x 128 threads).  partials holds `capacity` entries;
 // cudaErrorInvalidValue (nothing launched) if the pass needs more.

@@ -38,6 +38,7 @@
 
 #include "ah_internal.cuh"
 #include "diag_common.cuh"
+#include "diag_pair.cuh"
 #include "diag_tile.cuh"
 #include "sincos32.cuh"
 
@@ -401,16 +402,44 @@ __global__ void __launch_bounds__(256, MINB)
     t.flush(&da.partials[blockIdx.x]);
 }
 
+// The same on 32 x 16 columns, two rows per thread (diag_pair.cuh).
+template <typename IT>
+__global__ void __launch_bounds__(256, 2)
+    k_diag_pair(View<float> v, int N, int tx, int ty, int items, int zc, SiteCoef<float> sc, DiagArgs da)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    DiagPair<IT> t;
+    for (int it = blockIdx.x; it < items; it += gridDim.x) {
+        const int bx = it % tx, by = (it / tx) % ty, z0 = it / (tx * ty) * zc;
+        t.column(v, N, da, sc, 32 * bx, 16 * by, z0, min(z0 + zc, N), smem_raw);
+    }
+    t.flush(&da.partials[blockIdx.x]);
+}
+
 // CTAs per SM that the registers allow
 template <typename real> constexpr int kDiagCtas = sizeof(real) == 4 ? 2 : 1;
 
-struct DiagGrid { int tx, ty, zc, items, ctas; };
+struct DiagGrid { int tx, ty, zc, items, ctas; bool pair; };
+// FP32 lattices whose rows can be copied in 16 bytes take two rows per thread.
 template <typename real>
-DiagGrid diag_whole_grid(int N)
+bool diag_pair_ok(const View<real> &v, int N)
+{
+    if constexpr (sizeof(real) == 8) {
+        return false;
+    } else {
+        const void *const p[10] = { v.phr, v.phi, v.th1, v.th2, v.th3, v.pir, v.pii, v.e1, v.e2, v.e3 };
+        uintptr_t bits = 0;
+        for (const void *q : p) bits |= reinterpret_cast<uintptr_t>(q);
+        return feed_ok(N) && (bits & 15) == 0;
+    }
+}
+template <typename real>
+DiagGrid diag_whole_grid(const View<real> &v, int N)
 {
     DiagGrid g;
+    g.pair = diag_pair_ok(v, N);
     g.tx = (N + 31) / 32;
-    g.ty = (N + 7) / 8;
+    g.ty = g.pair ? (N + 15) / 16 : (N + 7) / 8;
     const int n = choose_chunks(N, (long long)g.tx * g.ty, kDiagCtas<real>, 1, PlaneTimes{ { 193, 255 } });
     g.zc = (N + n - 1) / n;
     g.items = g.tx * g.ty * ((N + g.zc - 1) / g.zc);
@@ -419,50 +448,60 @@ DiagGrid diag_whole_grid(int N)
 }
 
 template <typename real, typename IT>
-cudaError_t launch_diag_whole_it(const View<real> &v, int N, const DiagArgs &da, cudaStream_t st)
+cudaError_t launch_diag_whole_it(const View<real> &v, int N, const DiagGrid &g, const DiagArgs &da, cudaStream_t st)
 {
     constexpr size_t smem = DiagGeo::smem<real>;
     constexpr int minb = kDiagCtas<real>;
     static unsigned long long configured = 0;   // per device; dynamic plus static smem may pass 48 KB
     const unsigned long long dev_bit = 1ULL << device_slot();
     if (!(configured & dev_bit)) {
-        const cudaError_t e = cudaFuncSetAttribute(k_diag_whole<real, IT, minb>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(k_diag_whole<real, IT, minb>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)smem);
+        if (e == cudaSuccess && sizeof(real) == 4)
+            e = cudaFuncSetAttribute(k_diag_pair<IT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)DiagPairGeo::smem);
         if (e != cudaSuccess) return e;
         configured |= dev_bit;
     }
-    const DiagGrid g = diag_whole_grid<real>(N);
-    k_diag_whole<real, IT, minb><<<g.ctas, 256, smem, st>>>(v, N, g.tx, g.ty, g.items, g.zc, site_coef(da.dc, real(0)),
-                                                           da);
+    const SiteCoef<real> sc = site_coef(da.dc, real(0));
+    if constexpr (sizeof(real) == 4) {
+        if (g.pair) {
+            k_diag_pair<IT><<<g.ctas, 256, DiagPairGeo::smem, st>>>(v, N, g.tx, g.ty, g.items, g.zc, sc, da);
+            return cudaGetLastError();
+        }
+    }
+    k_diag_whole<real, IT, minb><<<g.ctas, 256, smem, st>>>(v, N, g.tx, g.ty, g.items, g.zc, sc, da);
     return cudaGetLastError();
 }
 }  // namespace
 
 int fused_diag_max_ctas() { return std::max(kDiagCtas<float>, kDiagCtas<double>) * device_sm_count(); }
 
+namespace {
 template <typename real>
-cudaError_t launch_fused_diag(const View<real> &v, int N, const DiagArgs &da, cudaStream_t st)
+cudaError_t launch_diag_grid(const View<real> &v, int N, const DiagGrid &g, const DiagArgs &da, cudaStream_t st)
 {
-    return (long long)N * N * N < (1LL << 31) ? launch_diag_whole_it<real, int>(v, N, da, st)
-                                              : launch_diag_whole_it<real, long long>(v, N, da, st);
+    return (long long)N * N * N < (1LL << 31) ? launch_diag_whole_it<real, int>(v, N, g, da, st)
+                                              : launch_diag_whole_it<real, long long>(v, N, g, da, st);
 }
+}  // namespace
 
 template <typename real>
 cudaError_t launch_diag_whole(const View<real> &v, int N, const DiagCoef &c, DiagPartial *partials,
                               int capacity, DiagPartial *result, DiagList list, int fix_blocks, cudaStream_t st)
 {
     // one partial per CTA of the tile walk: refuse a buffer that cannot hold them
-    const int ctas = diag_whole_grid<real>(N).ctas;
-    if (ctas > capacity) return cudaErrorInvalidValue;
+    const DiagGrid g = diag_whole_grid<real>(v, N);
+    if (g.ctas > capacity) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemsetAsync(list.count, 0, sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
     DiagArgs da;
     da.dc = c;
     da.partials = partials;
     da.list = list;
-    e = launch_fused_diag<real>(v, N, da, st);
+    e = launch_diag_grid<real>(v, N, g, da, st);
     if (e != cudaSuccess) return e;
-    return launch_diag_reduce<real>(v, N, partials, ctas, result, list, fix_blocks, st);
+    return launch_diag_reduce<real>(v, N, partials, g.ctas, result, list, fix_blocks, st);
 }
 
 template <typename real>
@@ -649,13 +688,13 @@ extern "C" ah_status ah_observables_noalloc(const float *const fields[10], int32
     da.dc = host_diag_coef(*cfg, step);
     da.partials = partials;
     da.list = list;
-    const int ctas = diag_whole_grid<float>(N).ctas;
-    if (ctas > kNoAllocBlocks)
+    const DiagGrid g = diag_whole_grid<float>(v, N);
+    if (g.ctas > kNoAllocBlocks)
         return host_fail(AH_ERR_CUDA, "ah_observables_noalloc: more resident CTAs than the scratch has partials");
     cudaError_t e = cudaMemsetAsync(list.count, 0, sizeof(unsigned long long), stream);
-    if (e == cudaSuccess) e = launch_fused_diag<float>(v, N, da, stream);
+    if (e == cudaSuccess) e = launch_diag_grid<float>(v, N, g, da, stream);
     if (e == cudaSuccess) {
-        k_diag_sum<<<1, 1024, 0, stream>>>(partials, ctas, result);
+        k_diag_sum<<<1, 1024, 0, stream>>>(partials, g.ctas, result);
         k_noalloc_fixup<float><<<nblocks, 128, 0, stream>>>(v, N, list, result);
         k_noalloc_wind_clear<<<1, 32, 0, stream>>>(list, result);
         k_noalloc_wind_all<float><<<nblocks, 256, 0, stream>>>(v, N, list, result);

@@ -47,7 +47,7 @@ def test_step_walk_matches_oracle(precision, N, th_amp):
 
 
 @pytest.mark.parametrize("th_amp", AMPLITUDES + [200.0])
-@pytest.mark.parametrize("precision,N", [(p, n) for p in (ah.AH_FP32, ah.AH_FP64) for n in (5, 31, 33, 42)])
+@pytest.mark.parametrize("precision,N", [(p, n) for p in (ah.AH_FP32, ah.AH_FP64) for n in (5, 31, 33, 42, 44)])
 def test_diagnostics_walk_matches_oracle(precision, N, th_amp):
     f = random_state(N, 11, th_amp=th_amp).astype(np.float32).astype(np.float64)
     with sim(N, precision, ah.AH_KERNEL_FUSED) as g:
