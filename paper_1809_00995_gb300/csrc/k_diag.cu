@@ -12,7 +12,8 @@
 //   2 pi W = Arg z1 + Arg z2 - Arg z3 - Arg z4 - Arg(z1 z2 conj(z3) conj(z4)),
 //   Arg in (-pi, pi] (the -pi branch value is mapped to +pi).
 //
-// Fast kernel (k_diag_fast): per-site energies in the state precision,
+// Box kernel (k_diag_fast; the whole lattice is walked by diag_tile.cuh and
+// diag_pair.cuh): per-site energies in the state precision,
 // accumulated per thread with compensated (Kahan) sums and reduced across the
 // block in FP64; the Gauss residual in FP64.  Windings by carries instead of
 // arctangents: for Args a, b in (-pi, pi], a + b = Arg(uv) + 2 pi c with c
@@ -29,7 +30,7 @@
 // Exact kernel (k_diag_exact): everything per site in FP64 with arctangents.
 //
 // Each block accumulates its sites in a fixed order and reduces with warp
-// shuffles; one block then adds the partials in index order, so the result
+// shuffles; k_diag_sum then adds the partials in a fixed order, so the result
 // depends only on the launch shape, never on scheduling (integer atomics of the
 // fix-up are order independent).
 #include <algorithm>
@@ -342,42 +343,37 @@ __global__ void __launch_bounds__(NT) k_diag_exact(View<real> v, int N, Box b, D
     block_reduce<NT>(acc, mx, ic, &partials[blockIdx.x]);
 }
 
-// Sum many partials in a fixed order: lane k of warp c reduces word k of
-// partials [c n/32, (c+1) n/32), then thread k adds the 32 chunk results.
-__global__ void __launch_bounds__(1024) k_diag_sum(const DiagPartial *partials, int n, DiagPartial *result)
+// Sum many partials in a fixed order: block k reduces word k, thread t the partials
+// t, t + 128, ..., then a tree over the threads.  Latency-bound: a chain of dependent
+// adds over strided loads, so its length is what counts (n / 128 adds and 7 levels;
+// one block with a warp per 1/32 of the partials had n / 32 + 32): 242 -> 229 us per
+// ah_observables_noalloc at 200^3.
+constexpr int kSumWords = kNumSums + kNumMax + kNumInt, kSumThreads = 128;
+__global__ void __launch_bounds__(kSumThreads) k_diag_sum(const DiagPartial *partials, int n, DiagPartial *result)
 {
-    constexpr int NW = kNumSums + kNumMax + kNumInt;
-    __shared__ double sd[32][kNumSums + kNumMax];
-    __shared__ long long si[32][kNumInt];
-    const int k = threadIdx.x & 31, c = threadIdx.x >> 5;
-    const int per = (n + 31) / 32, b0 = min(n, c * per), b1 = min(n, b0 + per);
-    if (k < kNumSums) {
-        double s = 0.0;
-        for (int b = b0; b < b1; ++b) s += partials[b].sums[k];
-        sd[c][k] = s;
-    } else if (k < kNumSums + kNumMax) {
-        double m = 0.0;
-        for (int b = b0; b < b1; ++b) m = fmax(m, partials[b].maxv[k - kNumSums]);
-        sd[c][k] = m;
-    } else if (k < NW) {
-        long long s = 0;
-        for (int b = b0; b < b1; ++b) s += partials[b].ints[k - kNumSums - kNumMax];
-        si[c][k - kNumSums - kNumMax] = s;
+    __shared__ double sd[kSumThreads];
+    __shared__ long long si[kSumThreads];
+    const int k = blockIdx.x, t = threadIdx.x;
+    double s = 0.0;
+    long long i = 0;
+    for (int b = t; b < n; b += kSumThreads) {
+        if (k < kNumSums) s += partials[b].sums[k];
+        else if (k < kNumSums + kNumMax) s = fmax(s, partials[b].maxv[k - kNumSums]);
+        else i += partials[b].ints[k - kNumSums - kNumMax];
     }
-    __syncthreads();
-    const int t = threadIdx.x;
-    if (t < kNumSums) {
-        double s = 0.0;
-        for (int q = 0; q < 32; ++q) s += sd[q][t];
-        result->sums[t] = s;
-    } else if (t < kNumSums + kNumMax) {
-        double m = 0.0;
-        for (int q = 0; q < 32; ++q) m = fmax(m, sd[q][t]);
-        result->maxv[t - kNumSums] = m;
-    } else if (t < NW) {
-        long long s = 0;
-        for (int q = 0; q < 32; ++q) s += si[q][t - kNumSums - kNumMax];
-        result->ints[t - kNumSums - kNumMax] = s;
+    sd[t] = s;
+    si[t] = i;
+    for (int o = kSumThreads / 2; o > 0; o >>= 1) {
+        __syncthreads();
+        if (t < o) {
+            sd[t] = k < kNumSums ? sd[t] + sd[t + o] : fmax(sd[t], sd[t + o]);
+            si[t] += si[t + o];
+        }
+    }
+    if (t == 0) {
+        if (k < kNumSums) result->sums[k] = sd[0];
+        else if (k < kNumSums + kNumMax) result->maxv[k - kNumSums] = sd[0];
+        else result->ints[k - kNumSums - kNumMax] = si[0];
     }
 }
 
@@ -508,7 +504,7 @@ template <typename real>
 cudaError_t launch_diag_reduce(const View<real> &v, int N, const DiagPartial *partials, int n, DiagPartial *result,
                                DiagList list, int fix_blocks, cudaStream_t st)
 {
-    k_diag_sum<<<1, 1024, 0, st>>>(partials, n, result);
+    k_diag_sum<<<kSumWords, kSumThreads, 0, st>>>(partials, n, result);
     k_diag_fixup<real><<<fix_blocks, 128, 0, st>>>(v, N, list, result);
     return cudaGetLastError();
 }
@@ -527,13 +523,13 @@ cudaError_t launch_diag(const View<real> &v, int N, Box b, const DiagCoef &c, Di
 {
     if (exact) {
         k_diag_exact<real><<<nblocks, NT, 0, st>>>(v, N, b, c, partials);
-        k_diag_sum<<<1, 1024, 0, st>>>(partials, nblocks, result);
+        k_diag_sum<<<kSumWords, kSumThreads, 0, st>>>(partials, nblocks, result);
         return cudaGetLastError();
     }
     cudaError_t e = cudaMemsetAsync(list.count, 0, sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
     k_diag_fast<real><<<nblocks, NT, 0, st>>>(v, N, b, c, partials, list);
-    k_diag_sum<<<1, 1024, 0, st>>>(partials, nblocks, result);
+    k_diag_sum<<<kSumWords, kSumThreads, 0, st>>>(partials, nblocks, result);
     k_diag_fixup<real><<<nblocks, 128, 0, st>>>(v, N, list, result);
     return cudaGetLastError();
 }
@@ -694,7 +690,7 @@ extern "C" ah_status ah_observables_noalloc(const float *const fields[10], int32
     cudaError_t e = cudaMemsetAsync(list.count, 0, sizeof(unsigned long long), stream);
     if (e == cudaSuccess) e = launch_diag_grid<float>(v, N, g, da, stream);
     if (e == cudaSuccess) {
-        k_diag_sum<<<1, 1024, 0, stream>>>(partials, g.ctas, result);
+        k_diag_sum<<<kSumWords, kSumThreads, 0, stream>>>(partials, g.ctas, result);
         k_noalloc_fixup<float><<<nblocks, 128, 0, stream>>>(v, N, list, result);
         k_noalloc_wind_clear<<<1, 32, 0, stream>>>(list, result);
         k_noalloc_wind_all<float><<<nblocks, 256, 0, stream>>>(v, N, list, result);
