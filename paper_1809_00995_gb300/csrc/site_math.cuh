@@ -30,16 +30,11 @@ __device__ __forceinline__ double two_sum_err(double a, double b, double s)
     return ad(sb(a, sb(s, bb)), sb(b, bb));
 }
 
-// U phi and conj(U) phi
+// U phi
 template <typename real>
 __device__ __forceinline__ V2<real> fwd(V2<real> u, V2<real> f)
 {
     return { fm(-u.i, f.i, ml(u.r, f.r)), fm(u.i, f.r, ml(u.r, f.i)) };
-}
-template <typename real>
-__device__ __forceinline__ V2<real> bwd(V2<real> u, V2<real> f)
-{
-    return { fm(u.i, f.i, ml(u.r, f.r)), fm(-u.i, f.r, ml(u.r, f.i)) };
 }
 
 // U = e^{i theta} of NL links of a site (sincos64.cuh; one warp vote picks the
@@ -105,15 +100,24 @@ __device__ __forceinline__ void plaq_sines(const double *ti, const double *tij, 
 }
 
 // One kick of Pi (Eq. up_pi) and the scalar currents Im[conj(U_d phi^{x+d}) phi^x]
-// of a site: f0 = phi^x, w_d = U_d phi^{x+d}, b_d = conj(U_d^{x-d}) phi^{x-d}.
+// of a site: f0 = phi^x, w_d = U_d phi^{x+d}; ub_d, fb_d the link and the field of
+// x - d, whose backward product conj(U) phi goes into the Laplacian by
+// multiply-adds.
 template <typename real>
 struct PiKick { real pr, pi, c1, c2, c3; };
 template <typename real>
 __device__ __forceinline__ PiKick<real> pi_kick(const KickCoef<real> &c, V2<real> f0, V2<real> w1, V2<real> w2,
-                                                V2<real> w3, V2<real> b1, V2<real> b2, V2<real> b3, real pr, real pi)
+                                                V2<real> w3, V2<real> ub1, V2<real> fb1, V2<real> ub2, V2<real> fb2,
+                                                V2<real> ub3, V2<real> fb3, real pr, real pi)
 {
-    const real lr = fm(real(-6), f0.r, ad(ad(ad(w1.r, b1.r), ad(w2.r, b2.r)), ad(w3.r, b3.r)));
-    const real li = fm(real(-6), f0.i, ad(ad(ad(w1.i, b1.i), ad(w2.i, b2.i)), ad(w3.i, b3.i)));
+    real lr = fm(real(-6), f0.r, ad(ad(w1.r, w2.r), w3.r));
+    real li = fm(real(-6), f0.i, ad(ad(w1.i, w2.i), w3.i));
+    lr = fm(ub1.i, fb1.i, fm(ub1.r, fb1.r, lr));
+    li = fm(-ub1.i, fb1.r, fm(ub1.r, fb1.i, li));
+    lr = fm(ub2.i, fb2.i, fm(ub2.r, fb2.r, lr));
+    li = fm(-ub2.i, fb2.r, fm(ub2.r, fb2.i, li));
+    lr = fm(ub3.i, fb3.i, fm(ub3.r, fb3.r, lr));
+    li = fm(-ub3.i, fb3.r, fm(ub3.r, fb3.i, li));
     const real pot = ml(c.c_pot, sb(fm(f0.r, f0.r, ml(f0.i, f0.i)), c.sigma2));
     PiKick<real> k;
     k.pr = fm(c.c_lap, lr, fm(-pot, f0.r, ml(c.c_damp, pr)));

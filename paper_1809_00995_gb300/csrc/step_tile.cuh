@@ -5,12 +5,11 @@
 // of its neighbours goes through shared memory in the form in which the
 // neighbour already has it:
 //   phi^{x+1}, phi^{x+y}                        forward products U_d phi^{x+d};
-//   conj(U_1) phi of x - 1, conj(U_2) phi of x - y   the backward products, formed
-//                                               by the site that owns the link;
+//   U_1, phi of x - 1 and U_2, phi of x - y     backward products conj(U) phi;
 //   theta_2, theta_3 of x + 1, theta_1, theta_3 of x + y   plaquette phases;
 //   sin Xi_12, sin Xi_13 of x - 1, sin Xi_12, sin Xi_23 of x - y   curls.
 // Plane z + 1 is in the thread's own registers (its loads are issued one plane
-// ahead) and of plane z - 1 only conj(U_3) phi and two sines are kept there.  One
+// ahead) and of plane z - 1 only U_3, phi and two sines are kept there.  One
 // buffer serves all planes, with two barriers per plane:
 //   B  (after the fields of plane z are in place)  plaquette sines to shared
 //      memory; Laplacian, Pi kick and phi drift, stored;
@@ -19,6 +18,14 @@
 // The halo ring needs link exponentials only where a link points into the tile
 // (theta_2 of the row below, theta_1 of the column to the left); the row above
 // and the column to the right are copies.
+//
+// What bounds it is the FP64 pipe, at 85 % of which nothing else matters: hence
+// links instead of backward products in the buffer (a product costs four FP64
+// instructions, its accumulation from link and field four as well, and the four
+// adds that it would need after that are saved), and nothing of plane z0 - 1 but
+// U_3 in the prologue.  One step at 256^3: 6.84 ms with plaquettes from products
+// of link exponentials, 5.4 ms with phases, 5.14 ms with links exchanged; 128^3
+// 0.665 ms, 64^3 0.113 ms.
 #pragma once
 #include "fused_common.cuh"
 #include "site_math.cuh"
@@ -31,7 +38,7 @@ struct TileGeo {
     static constexpr int TX = 32, NT = 32 * TY;
     static constexpr int EX = TX + 2, EY = TY + 2, NE = EX * EY;     // the tile and its ring
     // per site { phi.re, phi.im, theta_3, theta_2 }, then arrays of pairs (one
-    // address register serves them all): conj(U_1) phi, conj(U_2) phi,
+    // address register serves them all): U_1, U_2,
     // { sin 12, sin 13 }, { sin 12, sin 23 }, theta_1 (first of its pair)
     static constexpr size_t off_pairs = sizeof(V4<real>) * NE, stride = sizeof(V2<real>) * NE;
     static constexpr size_t smem = off_pairs + 5 * stride;
@@ -49,8 +56,8 @@ struct TileSite {
     {
         return *(reinterpret_cast<V2<real> *>(p + k * G::stride) + d);
     }
-    __device__ __forceinline__ V2<real> &b1(int d = 0) const { return pair(0, d); }
-    __device__ __forceinline__ V2<real> &b2(int d = 0) const { return pair(1, d); }
+    __device__ __forceinline__ V2<real> &u1(int d = 0) const { return pair(0, d); }
+    __device__ __forceinline__ V2<real> &u2(int d = 0) const { return pair(1, d); }
     __device__ __forceinline__ V2<real> &s1(int d = 0) const { return pair(2, d); }
     __device__ __forceinline__ V2<real> &s2(int d = 0) const { return pair(3, d); }
     __device__ __forceinline__ real &th1(int d = 0) const { return pair(4, d).r; }
@@ -105,6 +112,7 @@ __device__ __forceinline__ void step_tile(const View<real> &v, int N, int zc, co
     const TileSite<real, TY> R(smem_raw, h.e);
     const IT hoff = (IT)h.off;
 
+    auto field_of = [](const V4<real> &q) { return C{ q.a, q.b }; };
     // fields of the next plane: own site and ring site
     C fn, hf;
     real tn[3], ht[3];
@@ -118,39 +126,42 @@ __device__ __forceinline__ void step_tile(const View<real> &v, int N, int zc, co
             ht[0] = v.th1[r]; ht[1] = v.th2[r]; ht[2] = v.th3[r];
         }
     };
-    // fields of the plane that becomes the current one into shared memory
+    // the plane that becomes the current one: its fields into shared memory, then
+    // the link exponentials
     C f0, u[3];
     real t0[3];
-    auto put_own = [&]() {
-        link_exps<3>(t0, u);
+    auto put_fields = [&]() {
+        f0 = fn;
+        t0[0] = tn[0]; t0[1] = tn[1]; t0[2] = tn[2];
         S.field() = { f0.r, f0.i, t0[2], t0[1] };
         S.th1() = t0[0];
-        S.b1() = bwd(u[0], f0);
-        S.b2() = bwd(u[1], f0);
-    };
-    auto put_ring = [&]() {
         if (h.has) {
             R.field() = { hf.r, hf.i, ht[2], ht[1] };
             R.th1() = ht[0];
-            if (h.low) {
-                const real t = h.below ? ht[1] : ht[0];
-                C w;
-                link_exps<1>(&t, &w);
-                (h.below ? R.b2() : R.b1()) = bwd(w, hf);
-            }
         }
     };
+    auto put_ring_link = [&]() {
+        if (h.low) {
+            const real t = h.below ? ht[1] : ht[0];
+            C w;
+            link_exps<1>(&t, &w);
+            (h.below ? R.u2() : R.u1()) = w;
+        }
+    };
+    auto put_links = [&]() {
+        link_exps<3>(t0, u);
+        S.u1() = u[0];
+        S.u2() = u[1];
+    };
 
-    // prologue: of plane z0 - 1 only conj(U_3) phi and the sines of the two
-    // plaquettes that reach into plane z0
-    C b3;
+    // prologue: of plane z0 - 1 only U_3, phi and the sines of the two plaquettes
+    // that reach into plane z0
+    C um, fb;
     real p13m, p23m;
     load_plane((IT)(z0 == 0 ? N - 1 : z0 - 1) * plane);
-    f0 = fn;
-    t0[0] = tn[0]; t0[1] = tn[1]; t0[2] = tn[2];
-    put_own();
-    put_ring();
-    b3 = bwd(u[2], f0);
+    put_fields();
+    link_exps<1>(&t0[2], &um);
+    fb = f0;
     IT o0 = (IT)z0 * plane;                                   // planes z, z + 1, z + 2
     IT o1 = z0 + 1 == N ? 0 : o0 + plane;
     load_plane(o0);
@@ -164,9 +175,8 @@ __device__ __forceinline__ void step_tile(const View<real> &v, int N, int zc, co
         p23m = p[1];
     }
     __syncthreads();
-    f0 = fn;
-    t0[0] = tn[0]; t0[1] = tn[1]; t0[2] = tn[2];
-    put_ring();
+    put_fields();
+    put_ring_link();
     real pr, pim, e1, e2, e3;
     auto load_momenta = [&](IT base) {
         const IT s = base + roff;
@@ -175,7 +185,7 @@ __device__ __forceinline__ void step_tile(const View<real> &v, int N, int zc, co
     };
     load_plane(o1);
     load_momenta(o0);
-    put_own();
+    put_links();
 
     for (int z = z0;; ++z) {
         IT o2 = o1 + plane;
@@ -202,7 +212,8 @@ __device__ __forceinline__ void step_tile(const View<real> &v, int N, int zc, co
             (h.below ? R.s2() : R.s1()) = { ph[0], ph[1] };
         }
         const C w1 = fwd(u[0], C{ qx.a, qx.b }), w2 = fwd(u[1], C{ qy.a, qy.b }), w3 = fwd(u[2], fn);
-        const PiKick<real> k = pi_kick(c, f0, w1, w2, w3, S.b1(-1), S.b2(-EX), b3, pr, pim);
+        const PiKick<real> k = pi_kick(c, f0, w1, w2, w3, S.u1(-1), field_of(S.field(-1)), S.u2(-EX),
+                                       field_of(S.field(-EX)), um, fb, pr, pim);
         const real l1 = e_local(c, e1, k.c1), l2 = e_local(c, e2, k.c2), l3 = e_local(c, e3, k.c3);
         const real g1 = ad(p[0], sb(p[1], p13m)), g2 = sb(sb(p[2], p23m), p[0]), g3 = ad(p[1], p[2]);
         const IT s = o0 + roff;
@@ -212,7 +223,8 @@ __device__ __forceinline__ void step_tile(const View<real> &v, int N, int zc, co
             v.ophr[s] = fm(c.dt, k.pr, f0.r);
             v.ophi[s] = fm(c.dt, k.pi, f0.i);
         }
-        b3 = bwd(u[2], f0);
+        um = u[2];
+        fb = f0;
         p13m = p[1];
         p23m = p[2];
         __syncthreads();
@@ -233,12 +245,11 @@ __device__ __forceinline__ void step_tile(const View<real> &v, int N, int zc, co
         if (z + 1 == z1) break;
         o0 = o1;
         o1 = o2;
-        put_ring();                          // plane z + 1, before its registers are reloaded
-        f0 = fn;
-        t0[0] = tn[0]; t0[1] = tn[1]; t0[2] = tn[2];
+        put_fields();                        // plane z + 1, before its registers are reloaded
+        put_ring_link();
         load_plane(o1);
         load_momenta(o0);
-        put_own();
+        put_links();
     }
 }
 
