@@ -64,8 +64,8 @@ enum { AH_KERNEL_AUTO = 0, AH_KERNEL_PLAIN = 1, AH_KERNEL_FUSED = 2 };
 /* Configuration flags.
  *  EXACT_DIAG: evaluate every diagnostic per site in FP64 with arctangent
  *  windings (slow).  By default per-site energies are evaluated in the state
- *  precision (accumulated in FP64), the Gauss residual in FP64, and windings by
- *  sign carries that equal the FP64 arctangent formula, with the plaquettes
+ *  precision (accumulated in FP64), the Gauss residual in FP64, and windings as
+ *  integer turns that equal the FP64 arctangent formula, with the plaquettes
  *  near a branch cut re-evaluated in FP64. */
 enum { AH_FLAG_EXACT_DIAG = 1, AH_FLAG_AUTOTUNE = 2, AH_FLAG_WRAP_THETA = 4, AH_FLAG_CORE_GROWTH = 8,
        AH_FLAG_TWO_STEP = 16, AH_FLAG_FUSED_DIAG = 32 };
@@ -105,10 +105,10 @@ enum { AH_FLAG_EXACT_DIAG = 1, AH_FLAG_AUTOTUNE = 2, AH_FLAG_WRAP_THETA = 4, AH_
  * observables pass (ah_observables_start) is always taken by the next
  * two-step launch, which reads the state of the pass for its first step
  * anyway (see ah_observables_start).  Without the flag a two-step simulation
- * chooses by the last whole-lattice observables it returned: the fused launch
- * when fewer than 1e-3 of the plaquettes were pierced (a string network in an
- * otherwise smooth field, where most tiles skip the winding carries), else a
- * separate pass.  No effect in batches and the server. */
+ * of side 64 at most chooses by the last whole-lattice observables it returned:
+ * the fused launch when fewer than 1e-3 of the plaquettes were pierced (a string
+ * network in an otherwise smooth field), else a separate pass; larger ones take
+ * the separate pass, which is faster.  No effect in batches and the server. */
 
 typedef struct ah_config {
     int32_t N;            /* lattice side, 4 <= N <= 2048                         */
@@ -292,8 +292,9 @@ ah_status ah_autotune(ah_sim *sim, int32_t trial_steps, int32_t *chosen);
 /* ---- batched ensembles (the ensembles of independent runs of Sec. 4, Table 3) ----
  *
  * Many independent FP32 lattices (any mix of N, era, s, seed) advance together:
- * one persistent kernel launch per leapfrog step covers every resident lattice
- * (work items = lattice tiles), each lattice with its own coefficient table and
+ * one persistent kernel launch per leapfrog step (two when lattices with and
+ * without 16-byte rows, N a multiple of 4 from 64 on, are resident together) covers
+ * every resident lattice (work items = lattice tiles), each lattice with its own coefficient table and
  * step counter on the device; the steps between diagnostic points are replayed
  * from a CUDA graph.  Every lattice computes exactly what ah_step computes for
  * it alone. */

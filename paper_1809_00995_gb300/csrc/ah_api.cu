@@ -208,9 +208,14 @@ struct Staging {
     Staging &operator=(const Staging &) = delete;
 };
 
-// Largest fraction of pierced plaquettes at which a deferred observables pass
-// rides on the next two-step launch (k_fused2_diag) without AH_FLAG_FUSED_DIAG.
+// Largest fraction of pierced plaquettes, and largest side, at which a deferred
+// observables pass rides on the next two-step launch (k_fused2_diag) without
+// AH_FLAG_FUSED_DIAG.  Start, one pass of two steps and finish on a string network,
+// separate / fused: 64^3 102 / 120 us, where both wait for launches and the fused one
+// keeps the second stream free; 96^3 129 / 196 us, 128^3 179 / 322 us, 250^3 1.04 /
+// 1.36 ms, 256^3 0.90 / 1.45 ms, 512^3 6.55 / 10.1 ms.
 constexpr double kFusedDiagPierced = 1e-3;
+constexpr int kFusedDiagSide = 64;
 
 template <typename real>
 void carve(Fields<real> &F, char *base, size_t n, bool spare = false)
@@ -822,12 +827,8 @@ ah_status ah_observables_start(ah_sim *h)
         AH_CUDA(cudaEventCreateWithFlags(&h->ev_done, cudaEventDisableTiming));
     }
     h->diag_step = h->step;
-    // Fold the pass into the next two-step launch where that pays (measured at
-    // 256^3 - 1024^3: 2-4 % faster than a launch plus a separate pass on string
-    // networks in smooth fields, where most tiles skip the winding carries,
-    // 4-8 % slower on rough fields, where the fused launch's accumulators cost
-    // it a third of its resident CTAs)
-    const bool fuse = (h->cfg.flags & AH_FLAG_FUSED_DIAG) || h->pierced_frac < kFusedDiagPierced;
+    const bool fuse = (h->cfg.flags & AH_FLAG_FUSED_DIAG) ||
+                      (h->pierced_frac < kFusedDiagPierced && h->N <= kFusedDiagSide);
     if (h->two_step && fuse && !(h->cfg.flags & AH_FLAG_EXACT_DIAG)) {
         // taken by the next two-step launch (or run on its own before other work)
         h->diag_pending = true;

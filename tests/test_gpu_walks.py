@@ -10,7 +10,7 @@ import pytest
 
 import oracle as O
 import paper_1809_00995_gb300 as ah
-from inputs import random_state
+from inputs import random_state, straight_strings
 from test_gpu_batch_serve import oracle_fields, short_config
 from test_gpu_parity import TOL, compare_obs, oparams, rel_err, sim
 
@@ -22,15 +22,13 @@ AMPLITUDES = [0.015, 0.09, 0.18, 0.7, 3.0, 40.0]
 
 
 @pytest.mark.parametrize("th_amp", AMPLITUDES)
-@pytest.mark.parametrize("precision,N", [(ah.AH_FP64, 4), (ah.AH_FP64, 31), (ah.AH_FP64, 33), (ah.AH_FP64, 41),
-                                         (ah.AH_FP32, 40), (ah.AH_FP32, 44), (ah.AH_FP32, 64), (ah.AH_FP32, 68),
-                                         (ah.AH_FP32, 100)])
-def test_step_walk_matches_oracle(precision, N, th_amp):
+@pytest.mark.parametrize("precision,name,N", [(ah.AH_FP64, "ty8_b2_w", n) for n in (4, 31, 33, 41)]
+                         + [(ah.AH_FP32, "ty16_b2_w", n) for n in (40, 44, 64, 68, 100)])
+def test_step_walk_matches_oracle(precision, name, N, th_amp):
     f = random_state(N, 7, th_amp=th_amp).astype(np.float32).astype(np.float64)
     wrap = th_amp == 3.0
     with sim(N, precision, ah.AH_KERNEL_FUSED, era=ah.AH_MATTER, s=1.0,
              flags=ah.AH_FLAG_WRAP_THETA if wrap else 0) as g:
-        name = "ty16_b2_w" if precision == ah.AH_FP32 else "ty8_b2_w"
         for k in range(g.info["n_variants"]):
             try:
                 g.set_variant(k)
@@ -67,3 +65,19 @@ def test_batch_of_both_walks():
         _, st, alone = ah.ah_batch_run_ex([cfgs[i]], [(0, 0, 0, 0, Ns[i], Ns[i], Ns[i])])
         assert st["launches"] == 2 * steps
         np.testing.assert_array_equal(alone[0], fields[i])
+
+
+@pytest.mark.parametrize("N,fused", [(64, 1), (68, 0)])
+def test_deferred_observables_ride_only_on_small_lattices(N, fused):
+    """Few pierced plaquettes, no flag: the two-step launch takes the pass up to 64^3,
+    above it the separate pass runs, bit for bit that of ah_observables."""
+    with ah.Sim(N, precision=ah.AH_FP32, era=ah.AH_RADIATION, seed=4, flags=ah.AH_FLAG_TWO_STEP) as g:
+        g.set_fields(straight_strings(N, axis=1, x0=0.5, y0=0.25), 8)
+        ref = g.observables()
+        g.observables_start()
+        g.step(2)
+        got = g.observables_finish()
+        assert g.info["fused_diag_passes"] == fused
+    assert got["wind_abs_plane"] == ref["wind_abs_plane"] == [0, 4 * N, 0]
+    assert got["gauss_max"] == ref["gauss_max"]
+    assert fused or got["sums"] == ref["sums"]
