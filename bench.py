@@ -110,7 +110,7 @@ def peaks():
 
 # sources of the single-step and the two-step kernel: a traffic record is void
 # once any of its kernel's sources changes
-KERNEL_SOURCES = {"k_fused": ("k_fused.cu", "fused_common.cuh", "sincos32.cuh"),
+KERNEL_SOURCES = {"k_fused": ("k_fused.cu", "feed_tile.cuh", "pair_math.cuh", "fused_common.cuh", "sincos32.cuh"),
                   "k_fused2": ("k_fused2.cu", "k_fused2_tile.cuh", "fused_common.cuh", "sincos32.cuh")}
 
 
@@ -575,8 +575,8 @@ def main():
                        "parallelism": "replicas" if world > 1 else "single"},
             "hbm_gbs_effective": achieved,
             "roofline": roofline,
-            # the rest of a bench step: one whole-lattice diagnostics pass (k_fused_diag
-            # tile walk, ordered sum, near-cut fix-up) and its read-back to the host
+            # the rest of a bench step: one whole-lattice diagnostics pass (tile
+            # walk of k_diag.cu, ordered sum, near-cut fix-up) and its read-back to the host
             "diag_pass": {"ms_per_pass": (t_ms - step_ms) / a.steps, "share_of_time": 1.0 - step_ms / t_ms,
                           "bound": "issue (FP32 arithmetic of the estimators, windings and double-float "
                                    "Gauss residual; one read of the state)"},

@@ -2,8 +2,9 @@
 //
 // Both run many independent FP32 lattices (the paper's ensemble of runs with
 // different seeds, eras and s, Sec. 4 and Table 3) on one GPU with the batched
-// fused step of k_fused.cu: one persistent launch per step advances every
-// resident lattice, whatever its size, by one leapfrog step (Eqs. up_pi, up_E,
+// fused step of k_fused.cu: per step one persistent launch for the lattices of each
+// of the two tile walks (feed_lattice; one launch where all take the same) advances
+// every resident lattice, whatever its size, by one leapfrog step (Eqs. up_pi, up_E,
 // up_phi, up_A), each with its own coefficient table and step counter in device
 // memory.  With AH_BATCH_TWO_STEP the batched two-step pass of k_fused2.cu
 // advances every lattice by two steps per launch (temporal blocking; a round

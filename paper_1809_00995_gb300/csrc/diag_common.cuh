@@ -1,5 +1,5 @@
 // diag_common.cuh -- device helpers shared by the diagnostics kernels
-// (k_diag.cu) and the fused step's diagnostics mode (k_fused.cu).
+// (k_diag.cu) and the two-step pass that carries the diagnostics (k_fused2.cu).
 #pragma once
 
 #include <climits>

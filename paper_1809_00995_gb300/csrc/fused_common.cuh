@@ -1,8 +1,8 @@
 // fused_common.cuh -- pieces shared by the z-marching step kernels
 // (k_fused.cu: one step per pass; k_fused2.cu: two steps per pass): complex
 // arithmetic on link exponentials U = e^{i theta}, plaquette products, the
-// tile geometry with its one-site halo ring, row loads/stores, and the
-// wave-quantisation model that picks the number of z chunks.
+// tile geometry with its one-site halo ring, row loads/stores, and the rule that
+// picks the number of z chunks.
 #pragma once
 #include "ah_internal.cuh"
 
@@ -18,11 +18,11 @@ struct PlaneTimes { short t[4]; };
 // each CTA marching its chunk of zc = ceil(N / n) planes plus `extra` planes'
 // worth of prologue, so minimise (zc + extra) (whole waves x t[per_sm] + t[CTAs per
 // SM of the last wave]) over n.  Chunks go down to a single plane: a lattice that
-// cannot fill the GPU is bound by the march of one CTA (64^3, FP32 step: 4 chunks
-// 23.6 us, 32 chunks 10.3 us; 32^3, FP64 step: 2 chunks 236 us, 32
-// chunks 26.7 us).  The times matter in
-// between: 3 resident CTAs take less than 3/4 of the time of 4, so at 125^3 seven
-// chunks (39.5 us) beat the nine that fill the wave (41.0 us).
+// cannot fill the GPU is bound by the march of one CTA (64^3, one-site FP32 step: 4
+// chunks 23.6 us, 32 chunks 10.3 us; 32^3, FP64 step before step_tile.cuh: 2 chunks
+// 236 us, 32 chunks 26.7 us).  The times matter in between: 3 resident CTAs take
+// less than 3/4 of the time of 4, so at 125^3 seven chunks (39.5 us) beat the nine
+// that fill the wave (41.0 us).
 int choose_chunks(int N, long long tiles, int per_sm, int extra, const PlaneTimes &times);
 
 namespace {

@@ -19,12 +19,13 @@
 // state exactly once from DRAM; halo re-reads are served by L2.  Periodic
 // boundaries are applied in the index arithmetic.
 //
-// The same tile walk serves two kernels: k_fused (one lattice, one step) and
-// k_fused_batch (persistent CTAs over the tiles of many lattices).  FP64
-// lattices of the default shape run step_tile.cuh instead.  The shapes (tile height, sites per thread in x, resident
-// CTAs per SM) and the number of z chunks per column are chosen by the
-// autotuner; a chunk count that fills the last wave of CTAs matters because
-// each CTA marches a whole chunk.
+// That walk serves k_fused (one lattice, one step) and k_fused_batch (persistent
+// CTAs over the tiles of many lattices).  FP32 lattices whose rows can be copied in
+// 16 bytes run feed_tile.cuh instead (k_feed, k_feed_batch), FP64 lattices of the
+// default shape step_tile.cuh.  The shapes (tile height, sites per thread in x,
+// resident CTAs per SM) are chosen by the default of the size or by the autotuner,
+// the number of z chunks per column by choose_chunks: each CTA marches a whole
+// chunk, so a poorly filled last wave costs a whole march.
 #include "ah_internal.cuh"
 #include "sincos32.cuh"
 #include "fused_common.cuh"

@@ -84,9 +84,8 @@ __device__ __forceinline__ C2<float> edge2(cpx<float> fa, cpx<float> u, cpx<floa
 }
 
 // One thread's share of the whole-lattice diagnostics: the same per-site
-// terms, in the same order and precision, as the diagnostics pass of the
-// single-step tile walk (k_fused.cu, MODE_DIAG), so the two agree to FP32
-// rounding and the windings exactly.
+// terms and precision as the separate pass (diag_tile.cuh, diag_pair.cuh), so the
+// two agree to FP32 rounding, the windings exactly and max |G| bit for bit.
 struct Diag2Acc {
     // ah_obs.sums 3..13: K, |D phi|^2, V, E_el, B, K V, |D phi|^2 V, K L,
     // |D phi|^2 L, p L, rho L (compensated; the sums of L, rho, p follow)

@@ -21,11 +21,11 @@
 //
 // What bounds it is the FP64 pipe, at 85 % of which nothing else matters: hence
 // links instead of backward products in the buffer (a product costs four FP64
-// instructions, its accumulation from link and field four as well, and the four
+// instructions, its accumulation from link and field four as well, and the two
 // adds that it would need after that are saved), and nothing of plane z0 - 1 but
 // U_3 in the prologue.  One step at 256^3: 6.84 ms with plaquettes from products
-// of link exponentials, 5.4 ms with phases, 5.14 ms with links exchanged; 128^3
-// 0.665 ms, 64^3 0.113 ms.
+// of link exponentials, 5.4 ms with phases, 5.14 ms with links exchanged;
+// 128^3 0.665 ms, 64^3 0.113 ms.
 #pragma once
 #include "fused_common.cuh"
 #include "site_math.cuh"
