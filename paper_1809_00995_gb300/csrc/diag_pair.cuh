@@ -294,10 +294,8 @@ struct DiagPair : DiagTile<float, IT> {
                 auto count = [&](unsigned wm, unsigned wx, unsigned wy, unsigned wz, int row) {
                     const unsigned t = (0u - (wm + wx + wy + wz)) & 0xffffffu, cuts = (wm | wx | wy | wz) >> 24;
                     if (t | cuts) {
-                        const int w12 = (int)(t << 24) >> 24, r1 = (((int)(t << 8) >> 8) - w12) >> 8;
-                        const int w13 = (int)((unsigned)r1 << 24) >> 24;
-                        const int w23 = (int)((unsigned)((r1 - w13) >> 8) << 24) >> 24;
-                        const int q[3] = { w12, w13, w23 };
+                        int q[3];
+                        windings(t, q);
 #pragma unroll
                         for (int k = 0; k < 3; ++k) {
                             if (cuts >> k & 1u) {

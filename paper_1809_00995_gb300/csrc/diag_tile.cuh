@@ -74,10 +74,14 @@ __device__ __forceinline__ int turns(float a, bool *cut)
     *cut = !(fabsf(fmaf(-k, kTwoPi32, a)) <= kPi32 - kCutMargin);
     return __float_as_int(kb) - kRoundBits;
 }
+// k modulo 16, in [-8, 7].  Turns are counted modulo 16: a winding is at most 2, and
+// what the fields below add up, four links' turns (at most 8 each) and N, stays
+// within a field's 8 bits whatever the phases, so that a plaquette left to the FP64
+// list, whose sum lacks terms, borrows nothing from the next field.
+__device__ __forceinline__ int turns16(int k) { return (int)((unsigned)k << 28) >> 28; }
 // n_1, n_2, n_3 of a site's links to neighbours of phase b[], and a bit for each
-// that is too near the cut.  Phases past 8 give up their whole turns first, and
-// links with more than 24 turns count as near the cut, so that sums of four fit
-// the 8-bit fields below.
+// that is too near the cut.  Phases past 8 give up their whole turns first; links
+// with more than 24 turns count as near the cut.
 __device__ __forceinline__ int link_turns(float a, const float b[3], const float t[3], int n[3])
 {
     const float m = fmaxf(fabsf(t[0]), fmaxf(fabsf(t[1]), fabsf(t[2])));
@@ -92,7 +96,7 @@ __device__ __forceinline__ int link_turns(float a, const float b[3], const float
             const float r = fmaf(k, 1.74845553e-7f, fmaf(-k, 6.28318548f, t[d]));
             n[d] = turns(b[d] - a + r, &c[d]);
             c[d] = c[d] || !(fabsf(k) <= 24.f);
-            n[d] = c[d] ? 0 : n[d] + (int)k;
+            n[d] = c[d] ? 0 : turns16(n[d] + (int)k);
         }
     }
     if (!__any_sync(__activemask(), c[0] | c[1] | c[2])) return 0;
@@ -103,7 +107,7 @@ __device__ __forceinline__ int link_turns(float a, const float b[3], const float
 // The terms that a link's n adds to n_1 + n_2 - n_3 - n_4 of the plaquettes (12),
 // (13), (23), as three 8-bit fields (modulo 2^24) under three cut bits: of a site's
 // own links, of its links seen from x - 1 and from x - y, and from z - 1.  Words are
-// added, cut bits or-ed.
+// added, cut bits or-ed; windings takes the sum apart.
 __device__ __forceinline__ unsigned field_word(int v, int cut) { return ((unsigned)v & 0xffffffu) | (unsigned)cut << 24; }
 __device__ __forceinline__ unsigned own_word(const int n[3], int c)
 {
@@ -121,6 +125,16 @@ __device__ __forceinline__ unsigned y_word(int n1, int n3, int c)
 __device__ __forceinline__ unsigned z_word(const int n[3], int c)
 {
     return field_word(-n[0] * 256 - n[1] * 65536, c ? (c & 1) << 1 | (c >> 1 & 1) << 2 : 0);
+}
+// The three windings of a sum of words, N - (n_1 + n_2 - n_3 - n_4): fields are at most
+// 4 x 8 + 8 in size, so each is its low 8 bits with their sign.
+__device__ __forceinline__ void windings(unsigned t, int w[3])
+{
+    const int w12 = (int)(t << 24) >> 24, r1 = (((int)(t << 8) >> 8) - w12) >> 8;
+    const int w13 = (int)((unsigned)r1 << 24) >> 24;
+    w[0] = turns16(w12);
+    w[1] = turns16(w13);
+    w[2] = turns16((r1 - w13) >> 8);
 }
 
 // 1 - cos Xi summed over the three plaquettes of a site, from the four phases of
@@ -157,7 +171,7 @@ __device__ __forceinline__ float xi_terms(const float *ti, const float *tij, con
         const float r = fmaf(kf, 1.74845553e-7f, fmaf(-kf, 6.28318548f, d3.h)) + lo;
         const bool cut = !(fabsf(r) <= kPi32 - kCutMargin) || !(fabsf(kf) <= 96.f);
         cuts |= cut << k;
-        n -= cut ? 0 : (int)kf << 8 * k;
+        n -= cut ? 0 : turns16((int)kf) << 8 * k;
         float s, c;
         sincos_link(0.5f * r, &s, &c);
         sum = fmaf(2.f * s, s, sum);
@@ -189,7 +203,7 @@ __device__ __forceinline__ double xi_terms(const double *ti, const double *tij, 
         const float r = fmaf(kf, 1.74845553e-7f, fmaf(-kf, 6.28318548f, xf));
         const bool cut = !(fabsf(r) <= kPi32 - kCutMargin - 1e-6f * fabsf(kf)) || !(fabsf(kf) <= 96.f);
         cuts |= cut << k;
-        n -= cut ? 0 : (int)kf << 8 * k;
+        n -= cut ? 0 : turns16((int)kf) << 8 * k;
         double s, c;
         sincos_reduced(0.5 * x[k], 0.0, &s, &c);
         sum += 2.0 * s * s;
@@ -352,9 +366,8 @@ struct DiagTile {
                 const unsigned wx = atw(1 - b)[e + 1].x, wyv = atw(1 - b)[e + EX].y, wz = z_word(n, nc);
                 const unsigned t = (0u - (wm + wx + wyv + wz)) & 0xffffffu, cuts = (wm | wx | wyv | wz) >> 24;
                 if (t | cuts) {
-                    const int w12 = (int)(t << 24) >> 24, r1 = ((int)(t << 8) >> 8) - w12 >> 8;
-                    const int w13 = (int)((unsigned)r1 << 24) >> 24, w23 = (int)((unsigned)(r1 - w13 >> 8) << 24) >> 24;
-                    const int q[3] = { w12, w13, w23 };
+                    int q[3];
+                    windings(t, q);
 #pragma unroll
                     for (int k = 0; k < 3; ++k) {
                         if (cuts >> k & 1u) {

@@ -1,0 +1,39 @@
+"""Windings at link phases of many turns (GPU): the whole-lattice pass counts what the
+FP64 formula counts.  Sides of the one-row and of the
+two-row walk, each with ragged tiles."""
+import numpy as np
+import pytest
+
+import oracle as O
+import paper_1809_00995_gb300 as ah
+from inputs import random_state
+from test_gpu_parity import oparams, sim
+
+pytestmark = pytest.mark.gpu
+
+WALKS = [(p, n) for p in (ah.AH_FP32, ah.AH_FP64) for n in (33, 44)]
+TURN = 2 * np.pi
+
+
+def same_windings(N, precision, f, step):
+    f = f.astype(np.float32).astype(np.float64)
+    with sim(N, precision, ah.AH_KERNEL_FUSED) as g:
+        g.set_fields(f, step)
+        go = g.observables()
+    oo = O.observables(oparams(N), f, step)
+    assert list(go["wind_abs_plane"]) == list(oo["sum_abs_W_plane"])
+    assert list(go["wind_plane"]) == list(oo["sum_W_plane"])
+    assert go["n_pierced"] == oo["n_pierced"]
+
+
+@pytest.mark.parametrize("precision,N", WALKS)
+def test_turns_of_single_links_stay_in_their_plaquette(precision, N):
+    """A link of 150 turns in a plaquette of 90: the other plaquettes of the same
+    sites, whose links make tens of turns, keep their windings."""
+    f = random_state(N, 5, th_amp=0.0)
+    for z, y, x in [(5, 4, 3), (9, 15, 30), (N - 1, N - 1, N - 1)]:
+        xp, yp = (x + 1) % N, (y + 1) % N
+        f[5, z, y, xp] = 150 * TURN
+        f[4, z, y, x] = -20 * TURN
+        f[4, z, yp, x] = f[5, z, y, x] = 20 * TURN
+    same_windings(N, precision, f, 6)
