@@ -79,23 +79,43 @@ __device__ __forceinline__ int turns(float a, bool *cut)
 // within a field's 8 bits whatever the phases, so that a plaquette left to the FP64
 // list, whose sum lacks terms, borrows nothing from the next field.
 __device__ __forceinline__ int turns16(int k) { return (int)((unsigned)k << 28) >> 28; }
-// n_1, n_2, n_3 of a site's links to neighbours of phase b[], and a bit for each
-// that is too near the cut.  Phases past 8 give up their whole turns first; links
-// with more than 24 turns count as near the cut.
-__device__ __forceinline__ int link_turns(float a, const float b[3], const float t[3], int n[3])
+// t - 2 pi k, k the nearest integer of t / 2 pi (or its neighbour, where t / 2 pi rounds
+// across a half).  FP32 with 2 pi in two parts: up to 4 kMaxTurns turns the first
+// difference is exact and the second good to an ulp of pi.
+__device__ __forceinline__ float less_turns(float t, float *k)
 {
-    const float m = fmaxf(fabsf(t[0]), fmaxf(fabsf(t[1]), fabsf(t[2])));
+    *k = rintf(t * kInvTwoPi32);
+    return fmaf(*k, 1.74845553e-7f, fmaf(-*k, 6.28318548f, t));
+}
+__device__ __forceinline__ float less_turns(double t, float *k)
+{
+    const double kd = rint(t * 0.15915494309189535);
+    *k = (float)kd;
+    return (float)fma(-kd, 6.283185307179586, t);
+}
+// n_1, n_2, n_3 of a site's links to neighbours of phase b[], and a bit for each
+// that is too near the cut.  Phases past 8 give up their whole turns first.  Links
+// with more than kMaxTurns turns count as near the cut (and plaquettes with more than
+// four times as many), which sends all their plaquettes to the FP64 list: at 128^3,
+// random phases of up to 32 turns, a pass takes 0.13 ms, and 6.7 ms where the limit
+// lets the list overflow and every plaquette is counted again.
+constexpr float kMaxTurns = 4096.f;
+template <typename real>
+__device__ __forceinline__ int link_turns(float a, const float b[3], const real t[3], int n[3])
+{
+    const float f[3] = { (float)t[0], (float)t[1], (float)t[2] };
+    const float m = fmaxf(fabsf(f[0]), fmaxf(fabsf(f[1]), fabsf(f[2])));
     bool c[3];
     if (__all_sync(__activemask(), m <= 8.f)) {
 #pragma unroll
-        for (int d = 0; d < 3; ++d) n[d] = turns(b[d] - a + t[d], &c[d]);
+        for (int d = 0; d < 3; ++d) n[d] = turns(b[d] - a + f[d], &c[d]);
     } else {
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            const float k = rintf(t[d] * kInvTwoPi32);
-            const float r = fmaf(k, 1.74845553e-7f, fmaf(-k, 6.28318548f, t[d]));
+            float k;
+            const float r = less_turns(t[d], &k);
             n[d] = turns(b[d] - a + r, &c[d]);
-            c[d] = c[d] || !(fabsf(k) <= 24.f);
+            c[d] = c[d] || !(fabsf(k) <= kMaxTurns);
             n[d] = c[d] ? 0 : turns16(n[d] + (int)k);
         }
     }
@@ -166,10 +186,9 @@ __device__ __forceinline__ float xi_terms(const float *ti, const float *tij, con
     for (int k = 0; k < 3; ++k) {
         const DF d1 = two_sum(ti[k], -tij[k]), d2 = two_sum(tji[k], -tj[k]), d3 = two_sum(d1.h, d2.h);
         const float lo = d3.l + (d1.l + d2.l);
-        const float kf = rintf(d3.h * kInvTwoPi32);
-        // [Xi] = Xi - 2 pi k with 2 pi in two parts
-        const float r = fmaf(kf, 1.74845553e-7f, fmaf(-kf, 6.28318548f, d3.h)) + lo;
-        const bool cut = !(fabsf(r) <= kPi32 - kCutMargin) || !(fabsf(kf) <= 96.f);
+        float kf;
+        const float r = less_turns(d3.h, &kf) + lo;      // [Xi]
+        const bool cut = !(fabsf(r) <= kPi32 - kCutMargin) || !(fabsf(kf) <= 4.f * kMaxTurns);
         cuts |= cut << k;
         n -= cut ? 0 : turns16((int)kf) << 8 * k;
         float s, c;
@@ -199,9 +218,9 @@ __device__ __forceinline__ double xi_terms(const double *ti, const double *tij, 
     int n = 0, cuts = 0;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        const float xf = (float)x[k], kf = rintf(xf * kInvTwoPi32);
-        const float r = fmaf(kf, 1.74845553e-7f, fmaf(-kf, 6.28318548f, xf));
-        const bool cut = !(fabsf(r) <= kPi32 - kCutMargin - 1e-6f * fabsf(kf)) || !(fabsf(kf) <= 96.f);
+        float kf;
+        const float r = less_turns(x[k], &kf);           // [Xi]
+        const bool cut = !(fabsf(r) <= kPi32 - kCutMargin) || !(fabsf(kf) <= 4.f * kMaxTurns);
         cuts |= cut << k;
         n -= cut ? 0 : turns16((int)kf) << 8 * k;
         double s, c;
@@ -347,17 +366,17 @@ struct DiagTile {
             int n[3];
             int nc;
             {
-                const float bn[3] = { ax, ay, an }, tf[3] = { (float)t0[0], (float)t0[1], (float)t0[2] };
-                nc = link_turns(a0, bn, tf, n);
+                const float bn[3] = { ax, ay, an };
+                nc = link_turns(a0, bn, t0, n);
                 atw(b)[e] = make_uint2(x_word(n[1], n[2], nc), y_word(n[0], n[2], nc));
             }
             if (fwd) {
                 // the row above: n_1, n_3; the column to the right: n_2, n_3
                 const float rn = z < z1 ? site_phase((float)rf[0], (float)rf[1]) : 0.f;
                 const float aj = above ? atf(b)[he + 1] : (lx < 8 ? atf(b)[he + EX] : 0.f);
-                const float bn[3] = { aj, aj, rn }, tf[3] = { (float)g0[0], (float)g0[1], (float)g0[2] };
+                const float bn[3] = { aj, aj, rn };
                 int rk[3];
-                const int rc = link_turns(ra, bn, tf, rk);
+                const int rc = link_turns(ra, bn, g0, rk);
                 atw(b)[he] = make_uint2(x_word(rk[1], rk[2], rc), y_word(rk[0], rk[2], rc));
                 ra = rn;
             }

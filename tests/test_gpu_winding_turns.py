@@ -1,6 +1,8 @@
 """Windings at link phases of many turns (GPU): the whole-lattice pass counts what the
-FP64 formula counts.  Sides of the one-row and of the
+FP64 formula counts, and takes no longer for it.  Sides of the one-row and of the
 two-row walk, each with ragged tiles."""
+import time
+
 import numpy as np
 import pytest
 
@@ -37,3 +39,30 @@ def test_turns_of_single_links_stay_in_their_plaquette(precision, N):
         f[4, z, y, x] = -20 * TURN
         f[4, z, yp, x] = f[5, z, y, x] = 20 * TURN
     same_windings(N, precision, f, 6)
+
+
+# phases of up to 160, 1600, 4800 and 1.6e5 turns: within and past the limit of the walks' own count
+@pytest.mark.parametrize("th_amp", [1e3, 1e4, 3e4, 1e6])
+@pytest.mark.parametrize("precision,N", WALKS)
+def test_windings_at_many_turns(precision, N, th_amp):
+    same_windings(N, precision, random_state(N, 17, th_amp=th_amp), 6)
+
+
+@pytest.mark.parametrize("precision,N", [(ah.AH_FP32, 126), (ah.AH_FP32, 128), (ah.AH_FP64, 64)])
+def test_many_turns_take_no_recount(precision, N):
+    """Phases of up to 32 turns leave the plaquettes near a cut alone to the FP64
+    list: the pass takes about as long as with phases of half a turn (a recount of
+    every plaquette takes 8 times as long or more)."""
+    t = []
+    for th_amp in (3.0, 200.0):
+        with sim(N, precision, ah.AH_KERNEL_FUSED) as g:
+            g.set_fields(random_state(N, 3, th_amp=th_amp), 6)
+            g.observables()
+            runs = []
+            for _ in range(9):
+                t0 = time.perf_counter()
+                g.observables()
+                runs.append(time.perf_counter() - t0)
+            t.append(sorted(runs)[4])
+    print("\n%d^3, precision %d: %.0f us, %.0f us" % (N, precision, t[0] * 1e6, t[1] * 1e6))
+    assert t[1] <= 2.0 * t[0]
