@@ -67,13 +67,13 @@ __device__ __forceinline__ float2 site_phase2(float2 r, float2 i)
     p = fm(u, p, pk(-3.332567811012268e-01f));
     p = fm(u, p, pk(9.999992251396179e-01f));
     const float2 a = ml(q, p);
-    auto octant = [](float a, float r, float i, float x, float y, float hi, float lo) {
+    auto octant = [](float a, float r, float i, float x, float y, float hi) {
         a = y > x ? 0.5f * kPi32 - a : a;
         a = r < 0.f ? kPi32 - a : a;
         a = i < 0.f ? -a : a;
-        return hi > 1e-30f && hi < 1e30f && lo >= 0.f ? a : __int_as_float(0x7fc00000);
+        return hi > 1e-30f && x + y < 1e30f ? a : __int_as_float(0x7fc00000);
     };
-    return make_float2(octant(a.x, r.x, i.x, x.x, y.x, hi.x, lo.x), octant(a.y, r.y, i.y, x.y, y.y, hi.y, lo.y));
+    return make_float2(octant(a.x, r.x, i.x, x.x, y.x, hi.x), octant(a.y, r.y, i.y, x.y, y.y, hi.y));
 }
 
 // link_turns of both sites: n[d][row]; the cut bits of row 0, and of row 1 shifted by 3

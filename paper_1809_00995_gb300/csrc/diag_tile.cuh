@@ -53,6 +53,7 @@ __device__ __forceinline__ float atan_unit(float a)
     return a * p;
 }
 // arg phi to about 1e-6, or NaN where phi is too small, too large or not a number
+// (maximum and minimum pass over one NaN component, the sum does not)
 __device__ __forceinline__ float site_phase(float r, float i)
 {
     const float x = fabsf(r), y = fabsf(i), hi = fmaxf(x, y), lo = fminf(x, y);
@@ -60,7 +61,7 @@ __device__ __forceinline__ float site_phase(float r, float i)
     a = y > x ? 0.5f * kPi32 - a : a;
     a = r < 0.f ? kPi32 - a : a;
     a = i < 0.f ? -a : a;
-    return hi > 1e-30f && hi < 1e30f && lo >= 0.f ? a : __int_as_float(0x7fc00000);
+    return hi > 1e-30f && x + y < 1e30f ? a : __int_as_float(0x7fc00000);
 }
 
 // n of a link whose bracket is a - 2 pi n, and whether the bracket is too near
