@@ -330,7 +330,7 @@ struct DiagPair : DiagTile<float, IT> {
                 wm0 = ((w0 + wn[0]) & 0xffffffu) | ((w0 | wn[0]) & 0x07000000u);
                 wm1 = ((w1 + wn[1]) & 0xffffffu) | ((w1 | wn[1]) & 0x07000000u);
                 U22 u[3];
-                link_exps2<3, false>(t0, u);
+                link_exps2<3>(t0, u);
                 const C22 fx = { raw2(rb, 0, 1), raw2(rb, 1, 1) };
                 const C22 fy = { make_float2(f0r.y, raw(rb, 0, 2, 0)), make_float2(f0i.y, raw(rb, 1, 2, 0)) };
                 const C22 w1c = fwd(u[0], fx), w2c = fwd(u[1], fy), w3c = fwd(u[2], C22{ fnr, fni });

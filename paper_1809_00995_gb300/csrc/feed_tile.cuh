@@ -155,7 +155,7 @@ __device__ __forceinline__ void feed_tile(const VIEW &v, int N, int zc, const CO
         f0.i = raw2(off, 1, 0, 0);
 #pragma unroll
         for (int d = 0; d < 3; ++d) t0[d] = raw2(off, 2 + d, 0, 0);
-        link_exps2<3, false>(t0, u);
+        link_exps2<3>(t0, u);
         const C22 b1 = bwd(u[0], f0);
         *b1s = cat(b1.r, b1.i);
         b2 = bwd(u[1], f0);
@@ -163,13 +163,13 @@ __device__ __forceinline__ void feed_tile(const VIEW &v, int N, int zc, const CO
         if (wp == 0) {
             const float2 t = pk(rowb(off, 3, 0, 0));
             U22 w;
-            link_exps2<1, false>(&t, &w);
+            link_exps2<1>(&t, &w);
             const C22 b = bwd(w, C22{ pk(rowb(off, 0, 0, 0)), pk(rowb(off, 1, 0, 0)) });
             reinterpret_cast<float2 *>(smem + G::off_hb)[be] = make_float2(b.r.x, b.i.x);
         } else if (wp == 2 && lx < NP) {
             const float2 t = colb(off, 2, 0, 0);
             U22 w;
-            link_exps2<1, false>(&t, &w);
+            link_exps2<1>(&t, &w);
             const C22 b = bwd(w, C22{ colb(off, 0, 0, 0), colb(off, 1, 0, 0) });
             reinterpret_cast<float4 *>(smem + G::off_b1)[le] = cat(b.r, b.i);
         }
@@ -197,7 +197,7 @@ __device__ __forceinline__ void feed_tile(const VIEW &v, int N, int zc, const CO
         const float2 ti[2] = { t0[0], t0[1] }, tij[2] = { raw2(rb, 2, 0, 0), raw2(rb, 3, 0, 0) };
         const float2 tj[2] = { t0[2], t0[2] }, tji[2] = { raw2(ra, 4, 0, 1), raw2(ra, 4, 1, 0) };
         float2 p[2];
-        plaq_sines2<2, false>(ti, tij, tj, tji, p);
+        plaq_sines2<2>(ti, tij, tj, tji, p);
         p13m = p[0];
         p23m = p[1];
     }
@@ -227,7 +227,7 @@ __device__ __forceinline__ void feed_tile(const VIEW &v, int N, int zc, const CO
             const float2 tij[3] = { make_float2(t0[0].y, raw(rb, 2, 2, 0)), raw2(rc, 2, 0, 0), raw2(rc, 3, 0, 0) };
             const float2 tj[3] = { t0[1], t0[2], t0[2] };
             const float2 tji[3] = { raw2(rb, 3, 0, 1), raw2(rb, 4, 0, 1), make_float2(t0[2].y, raw(rb, 4, 2, 0)) };
-            plaq_sines2<3, false>(ti, tij, tj, tji, p);
+            plaq_sines2<3>(ti, tij, tj, tji, p);
             *s1s = cat(p[0], p[1]);
             *hps = make_float2(p[0].y, p[2].y);
         }
@@ -237,14 +237,14 @@ __device__ __forceinline__ void feed_tile(const VIEW &v, int N, int zc, const CO
             const float2 ti[2] = { t1, t2 }, tij[2] = { pk(rowb(rb, 2, 1, 0)), pk(rowb(rc, 3, 0, 0)) };
             const float2 tj[2] = { t2, t3 }, tji[2] = { pk(rowb(rb, 3, 0, 1)), pk(rowb(rb, 4, 1, 0)) };
             float2 q[2];
-            plaq_sines2<2, false>(ti, tij, tj, tji, q);
+            plaq_sines2<2>(ti, tij, tj, tji, q);
             reinterpret_cast<float2 *>(smem + G::off_hp)[be] = make_float2(q[0].x, q[1].x);
         } else if (wp == 3 && lx < NP) {
             const float2 t1 = colb(rb, 2, 0, 0), t2 = colb(rb, 3, 0, 0), t3 = colb(rb, 4, 0, 0);
             const float2 ti[2] = { t1, t1 }, tij[2] = { colb(rb, 2, 1, 0), colb(rc, 2, 0, 0) };
             const float2 tj[2] = { t2, t3 }, tji[2] = { colb(rb, 3, 0, 1), colb(rb, 4, 0, 1) };
             float2 q[2];
-            plaq_sines2<2, false>(ti, tij, tj, tji, q);
+            plaq_sines2<2>(ti, tij, tj, tji, q);
             reinterpret_cast<float4 *>(smem + G::off_s1)[le] = cat(q[0], q[1]);
         }
         float2 l1, l2, l3;

@@ -127,22 +127,14 @@ __device__ __forceinline__ float flip(float a, int bit1)   // -a if bit 1 of the
 }
 
 // U = e^{i theta} of NL links of both sites; one warp vote on the largest phase
-// picks the polynomials alone (|theta| <= 0.78; WEAK: the two-term forms where
-// |theta| <= 2^-6) or the reduced forms.
-template <int NL, bool WEAK>
+// picks the polynomials alone (|theta| <= 0.78) or the reduced forms.
+template <int NL>
 __device__ __forceinline__ void link_exps2(const float2 *t, U22 *u)
 {
     float m = amax2(t[0]);
 #pragma unroll
     for (int d = 1; d < NL; ++d) m = fmaxf(m, amax2(t[d]));
-    if (WEAK && __all_sync(__activemask(), m <= 0x1p-6f)) {
-#pragma unroll
-        for (int d = 0; d < NL; ++d) {
-            const float2 r2 = ml(t[d], t[d]);
-            u[d].i = fm(ml(t[d], r2), pk(-1.666666716e-01f), t[d]);
-            u[d].r = fm(r2, pk(-0.5f), pk(1.f));
-        }
-    } else if (__all_sync(__activemask(), m <= 0.78f)) {
+    if (__all_sync(__activemask(), m <= 0.78f)) {
 #pragma unroll
         for (int d = 0; d < NL; ++d) {
             u[d].i = sin_poly2(t[d]);
@@ -174,7 +166,7 @@ __device__ __forceinline__ void link_exps2(const float2 *t, U22 *u)
 // largest difference and the odd polynomial applies; beyond, the sum's rounding
 // errors (Knuth's TwoSum) are added after the range reduction, so that a Xi near
 // a multiple of 2 pi loses nothing.
-template <int NX, bool WEAK>
+template <int NX>
 __device__ __forceinline__ void plaq_sines2(const float2 *ti, const float2 *tij, const float2 *tj, const float2 *tji,
                                             float2 *p)
 {
@@ -185,13 +177,7 @@ __device__ __forceinline__ void plaq_sines2(const float2 *ti, const float2 *tij,
         x[k] = ad(sb(ti[k], tij[k]), sb(tji[k], tj[k]));
         m = k ? fmaxf(m, amax2(x[k])) : amax2(x[k]);
     }
-    if (WEAK && __all_sync(__activemask(), m <= 0x1p-4f)) {
-#pragma unroll
-        for (int k = 0; k < NX; ++k) {
-            const float2 r2 = ml(x[k], x[k]);
-            p[k] = fm(ml(x[k], r2), fm(r2, pk(8.333333768e-03f), pk(-1.666666716e-01f)), x[k]);
-        }
-    } else if (__all_sync(__activemask(), m <= 0.78f)) {
+    if (__all_sync(__activemask(), m <= 0.78f)) {
 #pragma unroll
         for (int k = 0; k < NX; ++k) p[k] = sin_poly2(x[k]);
     } else {
