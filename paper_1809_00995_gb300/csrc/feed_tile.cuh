@@ -194,12 +194,18 @@ __device__ __forceinline__ void feed_tile(const VIEW &v, int N, int zc, const CO
     C22 b3 = bwd(u[2], f0);
     float2 p13m, p23m;
     {
-        const float2 ti[2] = { t0[0], t0[1] }, tij[2] = { raw2(rb, 2, 0, 0), raw2(rb, 3, 0, 0) };
-        const float2 tj[2] = { t0[2], t0[2] }, tji[2] = { raw2(ra, 4, 0, 1), raw2(ra, 4, 1, 0) };
-        float2 p[2];
-        plaq_sines2<2>(ti, tij, tj, tji, p);
-        p13m = p[0];
-        p23m = p[1];
+        // all three plaquettes of plane z0 - 1, though only two of the sines are wanted:
+        // the vote in plaq_sines2 has to be the one that the loop takes for this plane,
+        // or the bits of plane z0 would depend on where the chunks begin (which, in a
+        // batch, the other lattices decide)
+        const float2 ti[3] = { t0[0], t0[0], t0[1] };
+        const float2 tij[3] = { make_float2(t0[0].y, raw(ra, 2, 2, 0)), raw2(rb, 2, 0, 0), raw2(rb, 3, 0, 0) };
+        const float2 tj[3] = { t0[1], t0[2], t0[2] };
+        const float2 tji[3] = { raw2(ra, 3, 0, 1), raw2(ra, 4, 0, 1), make_float2(t0[2].y, raw(ra, 4, 2, 0)) };
+        float2 p[3];
+        plaq_sines2<3>(ti, tij, tj, tji, p);
+        p13m = p[1];
+        p23m = p[2];
     }
     take_plane(rb);
 
