@@ -77,18 +77,19 @@ __device__ __forceinline__ double vers_range(double r)
     const double u = __dmul_rn(r, r);
     return __dmul_rn(u, __fma_rn(u, -cos_series<R>(u), 0.5));
 }
-static __device__ __noinline__ double2 sincos_far(double t)
+static __device__ __noinline__ double2 sincos_far64(double t)
 {
     double2 r;
     sincos(t, &r.x, &r.y);
     return r;
 }
 // sin, cos of t + lo, |lo| small beside |t| (the rounding error of a sum that
-// gave t; 0 for a phase taken as it is)
+// gave t; 0 for a phase taken as it is).  Without FAR |t| < 2^20 is the caller's to see to.
+template <bool FAR = true>
 __device__ __forceinline__ void sincos_reduced(double t, double lo, double *s, double *c)
 {
-    if (!(fabs(t) < 1048576.0)) {
-        const double2 r = sincos_far(t);
+    if (FAR && !(fabs(t) < 1048576.0)) {
+        const double2 r = sincos_far64(t);
         *s = r.x;
         *c = r.y;
         return;
@@ -112,5 +113,6 @@ __device__ __forceinline__ int abs_hi3(const double t[3]) { return max(abs_hi(t[
 constexpr int kHi2m4 = 0x3faffffe;       // just below 2^-4
 constexpr int kHi04 = 0x3fd99998;        // just below 0.4
 constexpr int kHi078 = 0x3fe8f5c1;       // just below 0.78
+constexpr int kHi2p18 = 0x41100000;      // 2^18
 
 }  // namespace ah

@@ -61,24 +61,37 @@ __device__ __forceinline__ void link_exps(const double *t, V2<double> *u)
     }
 }
 
+// sin Xi from the link exponentials, whose accuracy does not depend on the phases' size
+static __device__ __noinline__ double plaq_far(double ti, double tij, double tj, double tji)
+{
+    const double2 a = sincos_far64(ti), b = sincos_far64(tji), c = sincos_far64(tij), d = sincos_far64(tj);
+    const double abr = a.y * b.y - a.x * b.x, abi = a.y * b.x + a.x * b.y;
+    const double cdr = c.y * d.y - c.x * d.x, cdi = c.y * d.x + c.x * d.y;
+    return abi * cdr - abr * cdi;
+}
 // Sines of NX plaquettes from their phases: Xi = (ti - tij) + (tji - tj), the
-// phases of U_i^x, U_i^{x+j}, U_j^{x+i}, U_j^x.  When every |Xi| of the warp is
-// small the sum is good to an ulp of its largest difference and the odd
-// polynomial applies; beyond, the sum's rounding errors are kept (Knuth's
-// TwoSum) and added after the range reduction, so that a Xi near a multiple of
-// 2 pi (compact phases on the two sides of the cut) loses nothing.
+// phases of U_i^x, U_i^{x+j}, U_j^{x+i}, U_j^x.  Where |Xi| and |ti - tij| are at most
+// 0.78 for the whole warp the sum is good to 1.2 x 2^-53, as good as the links it is
+// made of, and the odd polynomial applies.  Beyond, the sum's rounding errors
+// (Knuth's TwoSum) are added after the range reduction: a Xi near a multiple of
+// 2 pi (compact phases on the two sides of the cut) and a small Xi between large phases
+// lose nothing.  Differences past 2^18, whose errors are no longer small, go through
+// the link exponentials (by a vote too, as calls among the reduced forms take
+// registers that the step has none of).
 template <int NX>
 __device__ __forceinline__ void plaq_sines(const double *ti, const double *tij, const double *tj, const double *tji,
                                            double *p)
 {
     double x[NX];
-    int m = 0;
+    int m = 0, ma = 0;
 #pragma unroll
     for (int k = 0; k < NX; ++k) {
-        x[k] = ad(sb(ti[k], tij[k]), sb(tji[k], tj[k]));
+        const double a = sb(ti[k], tij[k]);
+        x[k] = ad(a, sb(tji[k], tj[k]));
         m = max(m, abs_hi(x[k]));
+        ma = max(ma, abs_hi(a));
     }
-    const unsigned mm = __reduce_max_sync(__activemask(), (unsigned)m);
+    const unsigned mm = __reduce_max_sync(__activemask(), (unsigned)(ma <= kHi078 ? m : max(m, ma)));
     if (mm <= kHi2m4) {
 #pragma unroll
         for (int k = 0; k < NX; ++k) p[k] = sin_range<0>(x[k]);
@@ -88,13 +101,16 @@ __device__ __forceinline__ void plaq_sines(const double *ti, const double *tij, 
     } else if (mm <= kHi078) {
 #pragma unroll
         for (int k = 0; k < NX; ++k) p[k] = sin_range<2>(x[k]);
+    } else if (mm >= kHi2p18) {
+#pragma unroll
+        for (int k = 0; k < NX; ++k) p[k] = plaq_far(ti[k], tij[k], tj[k], tji[k]);
     } else {
 #pragma unroll
         for (int k = 0; k < NX; ++k) {
             const double a = sb(ti[k], tij[k]), b = sb(tji[k], tj[k]);
             const double ea = two_sum_err(ti[k], -tij[k], a), eb = two_sum_err(tji[k], -tj[k], b);
             double c;
-            sincos_reduced(x[k], ad(two_sum_err(a, b, x[k]), ad(ea, eb)), &p[k], &c);
+            sincos_reduced<false>(x[k], ad(two_sum_err(a, b, x[k]), ad(ea, eb)), &p[k], &c);
         }
     }
 }

@@ -155,7 +155,8 @@ __device__ __forceinline__ void step_tile(const View<real> &v, int N, int zc, co
     };
 
     // prologue: of plane z0 - 1 only U_3, phi and the sines of the two plaquettes
-    // that reach into plane z0
+    // that reach into plane z0 (whose votes are over fewer phases than the loop's: the
+    // last bits of a plane depend on where the chunks begin, which N and the GPU decide)
     C um, fb;
     real p13m, p23m;
     load_plane((IT)(z0 == 0 ? N - 1 : z0 - 1) * plane);
