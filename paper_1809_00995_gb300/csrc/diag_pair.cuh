@@ -123,8 +123,9 @@ __device__ __forceinline__ float2 xi_terms2(const float2 *ti, const float2 *tij,
     float m = 0.f;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        x[k] = ad(sb(ti[k], tij[k]), sb(tji[k], tj[k]));
-        m = fmaxf(m, amax2(x[k]));
+        const float2 a = sb(ti[k], tij[k]);
+        x[k] = ad(a, sb(tji[k], tj[k]));
+        m = fmaxf(fmaxf(m, amax2(a)), amax2(x[k]));
     }
     word[0] = word[1] = 0;
     if (__all_sync(__activemask(), m <= 0.78f)) {

@@ -31,7 +31,7 @@
 #include "diag_common.cuh"
 #include "fused_common.cuh"
 #include "sincos32.cuh"
-#include "sincos64.cuh"
+#include "site_math.cuh"
 
 namespace ah {
 namespace {
@@ -160,15 +160,39 @@ __device__ __forceinline__ void windings(unsigned t, int w[3])
 
 // 1 - cos Xi summed over the three plaquettes of a site, from the four phases of
 // each (as in Eq. 3: ti, tj at x, tij = theta_i^{x+j}, tji = theta_j^{x+i}); *word
-// the whole turns -N of each and the plaquettes whose [Xi] is too near the cut
+// the whole turns -N of each and the plaquettes whose [Xi] is too near the cut.  As in
+// the steps' plaq_sines the sum's rounding errors are kept unless |Xi| and |ti - tij|
+// are small for the whole warp, and the energies (the turns come with cut links) of
+// differences past 2^15 (FP64: 2^18) are those of the link exponentials.
+static __device__ __noinline__ float vers_far(float ti, float tij, float tj, float tji)
+{
+    C2<float> a, b, c, d;
+    sincosf(ti, &a.i, &a.r);
+    sincosf(tji, &b.i, &b.r);
+    sincosf(tij, &c.i, &c.r);
+    sincosf(tj, &d.i, &d.r);
+    const C2<float> z = cmul(cmul(a, b), conj(cmul(c, d)));
+    return one_minus_cos(z.r, z.i);
+}
+static __device__ __noinline__ double vers_far(double ti, double tij, double tj, double tji)
+{
+    C2<double> a, b, c, d;
+    sincos(ti, &a.i, &a.r);
+    sincos(tji, &b.i, &b.r);
+    sincos(tij, &c.i, &c.r);
+    sincos(tj, &d.i, &d.r);
+    const C2<double> z = cmul(cmul(a, b), conj(cmul(c, d)));
+    return one_minus_cos(z.r, z.i);
+}
 __device__ __forceinline__ float xi_terms(const float *ti, const float *tij, const float *tj, const float *tji,
                                           unsigned *word)
 {
     float x[3], m = 0.f, sum = 0.f;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        x[k] = (ti[k] - tij[k]) + (tji[k] - tj[k]);
-        m = fmaxf(m, fabsf(x[k]));
+        const float a = ti[k] - tij[k];
+        x[k] = a + (tji[k] - tj[k]);
+        m = fmaxf(m, fmaxf(fabsf(a), fabsf(x[k])));
     }
     *word = 0;
     if (__all_sync(__activemask(), m <= 0.78f)) {
@@ -196,6 +220,11 @@ __device__ __forceinline__ float xi_terms(const float *ti, const float *tij, con
         sincos_link(0.5f * r, &s, &c);
         sum = fmaf(2.f * s, s, sum);
     }
+    if (__any_sync(__activemask(), m >= 32768.f)) {
+        sum = 0.f;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) sum += vers_far(ti[k], tij[k], tj[k], tji[k]);
+    }
     *word = field_word(n, cuts);
     return sum;
 }
@@ -203,14 +232,16 @@ __device__ __forceinline__ double xi_terms(const double *ti, const double *tij, 
                                            unsigned *word)
 {
     double x[3], sum = 0.0;
-    int m = 0;
+    int m = 0, ma = 0;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        x[k] = (ti[k] - tij[k]) + (tji[k] - tj[k]);
+        const double a = sb(ti[k], tij[k]);
+        x[k] = ad(a, sb(tji[k], tj[k]));
         m = max(m, abs_hi(x[k]));
+        ma = max(ma, abs_hi(a));
     }
     *word = 0;
-    const unsigned mm = __reduce_max_sync(__activemask(), (unsigned)m);
+    const unsigned mm = __reduce_max_sync(__activemask(), (unsigned)(ma <= kHi078 ? m : max(m, ma)));
     if (mm <= kHi04) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) sum += mm <= kHi2m4 ? vers_range<0>(x[k]) : vers_range<1>(x[k]);
@@ -224,9 +255,16 @@ __device__ __forceinline__ double xi_terms(const double *ti, const double *tij, 
         const bool cut = !(fabsf(r) <= kPi32 - kCutMargin) || !(fabsf(kf) <= 4.f * kMaxTurns);
         cuts |= cut << k;
         n -= cut ? 0 : turns16((int)kf) << 8 * k;
+        const double a = sb(ti[k], tij[k]), b = sb(tji[k], tj[k]);
+        const double ea = two_sum_err(ti[k], -tij[k], a), eb = two_sum_err(tji[k], -tj[k], b);
         double s, c;
-        sincos_reduced(0.5 * x[k], 0.0, &s, &c);
+        sincos_reduced(0.5 * x[k], 0.5 * ad(two_sum_err(a, b, x[k]), ad(ea, eb)), &s, &c);
         sum += 2.0 * s * s;
+    }
+    if (mm >= kHi2p18) {
+        sum = 0.0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) sum += vers_far(ti[k], tij[k], tj[k], tji[k]);
     }
     *word = field_word(n, cuts);
     return sum;

@@ -1,6 +1,6 @@
 """Weak plaquettes between large link phases (GPU): Xi is a small difference of large
-phases (a gauge-rotated or long non-compact run), and its sine comes out as for small
-phases.  The reference is the phases' own exact sum in extended
+phases (a gauge-rotated or long non-compact run), and its sine and 1 - cos Xi come
+out as for small phases.  The reference is the phases' own exact sum in extended
 precision."""
 import numpy as np
 import pytest
@@ -56,3 +56,27 @@ def test_curl_of_weak_plaquettes(precision, N, amp, units):
     err = float(np.max(np.abs(e / c + curl)))
     print("\namp %g: %.2f units" % (amp, err / unit))
     assert err <= units * unit
+
+
+# 1 - cos Xi = Xi^2 / 2: twice the relative error of Xi, which is that of the kept sums (3
+# units), the polynomial and the coefficient (3 units), sums of positive terms
+# compensated (FP32) or 200 terms deep (FP64).
+@pytest.mark.parametrize("amp", [40.0, 3e3])
+@pytest.mark.parametrize("precision,N,tol", [(ah.AH_FP32, 33, 2.0 ** -20), (ah.AH_FP32, 44, 2.0 ** -20),
+                                             (ah.AH_FP64, 33, 2.0 ** -44), (ah.AH_FP64, 44, 2.0 ** -44)])
+def test_magnetic_energy_of_a_rounded_pure_gauge(precision, N, tol, amp):
+    """Every Xi is the rounding of its four phases, which the sum has to resolve; radiation
+    era, s = 0, e0 = 1: B = dx^-4 sum (1 - cos Xi)."""
+    f = np.zeros((10, N, N, N))
+    f[0] = 1.0
+    f[4:7] = links(N, amp, 0.0, 9)
+    if precision == ah.AH_FP32:
+        f = f.astype(np.float32).astype(np.float64)
+    with sim(N, precision, ah.AH_KERNEL_FUSED) as g:
+        g.set_fields(f, 6)
+        got = g.observables()["sums"][7]
+        dx = g.cfg.dx
+    xi = plaquettes(f[4:7])
+    ref = float(sum(np.sum(2 * np.sin(x / 2) ** 2) for x in xi.values())) / dx ** 4
+    print("\namp %g: %.3g, relative error %.3g" % (amp, ref, got / ref - 1))
+    assert abs(got - ref) <= tol * ref
