@@ -134,23 +134,18 @@ __device__ __forceinline__ DF df_mul(DF a, DF b)
 }
 // Gauss residual G = g_div div E + g_phi Im(conj(phi) Pi) of FP32 fields (div E from
 // E_d and E_d^{x-d}) to about 2^-44 of scale = |g_div div E| + |g_phi Im(...)|: the
-// differences and products of FP32 values are exact as pairs, high parts are
-// added with their errors (TwoSum), low parts in FP32.
+// differences and products of FP32 values are exact as pairs, and every sum and
+// product of pairs is brought back to a pair, so that a div E which is a small
+// difference of large E keeps its digits.  (Low parts added up once at the end save
+// a quarter of the instructions, but lose up to 2^-31 of scale.)
 struct GaussTerms { DF g; float scale; };
 __device__ __forceinline__ GaussTerms gauss_terms(DF g_div, DF g_phi, float fr, float fi, float pr, float pi, float e1,
                                                   float e1b, float e2, float e2b, float e3, float e3b)
 {
-    const DF d1 = two_sum(e1, -e1b), d2 = two_sum(e2, -e2b), d3 = two_sum(e3, -e3b);
-    const DF s1 = two_sum(d1.h, d2.h), s2 = two_sum(s1.h, d3.h);
-    const float sl = __fadd_rn(__fadd_rn(s1.l, s2.l), __fadd_rn(__fadd_rn(d1.l, d2.l), d3.l));
+    const DF div = df_add(df_add(two_sum(e1, -e1b), two_sum(e2, -e2b)), two_sum(e3, -e3b));
     const DF a = two_prod(fr, pi), b = two_prod(fi, pr);
-    const DF c = two_sum(a.h, -b.h);
-    const float cl = __fadd_rn(c.l, __fsub_rn(a.l, b.l));
-    const DF p = two_prod(g_div.h, s2.h), q = two_prod(g_phi.h, c.h);
-    const float pl = __fadd_rn(p.l, __fmaf_rn(g_div.h, sl, __fmul_rn(g_div.l, s2.h)));
-    const float ql = __fadd_rn(q.l, __fmaf_rn(g_phi.h, cl, __fmul_rn(g_phi.l, c.h)));
-    const DF g = two_sum(p.h, q.h);
-    return { fast_two_sum(g.h, __fadd_rn(g.l, __fadd_rn(pl, ql))), __fadd_rn(fabsf(p.h), fabsf(q.h)) };
+    const DF p = df_mul(g_div, div), q = df_mul(g_phi, df_add(a, { -b.h, -b.l }));
+    return { df_add(p, q), __fadd_rn(fabsf(p.h), fabsf(q.h)) };
 }
 __host__ __device__ __forceinline__ DF df_from(double x)
 {

@@ -33,25 +33,31 @@ __device__ __forceinline__ DF2 two_prod2(float2 a, float2 b)
     const float2 p = ml(a, b);
     return { p, fm(a, b, ng(p)) };
 }
+__device__ __forceinline__ DF2 df_add2(DF2 a, DF2 b)
+{
+    const DF2 s = two_sum2(a.h, b.h);
+    return two_sum2(s.h, ad(s.l, ad(a.l, b.l)));
+}
+__device__ __forceinline__ DF2 df_sub2(DF2 a, DF2 b)              // df_add(a, -b)
+{
+    const DF2 s = two_diff2(a.h, b.h);
+    return two_sum2(s.h, ad(s.l, sb(a.l, b.l)));
+}
+__device__ __forceinline__ DF2 df_mul2(DF a, DF2 b)
+{
+    const DF2 p = two_prod2(pk(a.h), b.h);
+    const float2 t = ad(p.l, fm(pk(a.h), b.l, ml(pk(a.l), b.h))), h = ad(p.h, t);
+    return { h, sb(t, sb(h, p.h)) };
+}
 struct GaussTerms2 { DF2 g; float2 scale; };
 __device__ __forceinline__ float2 abs2(float2 a) { return make_float2(fabsf(a.x), fabsf(a.y)); }
 __device__ __forceinline__ GaussTerms2 gauss_terms2(DF g_div, DF g_phi, float2 fr, float2 fi, float2 pr, float2 pi,
                                                     float2 e1, float2 e1b, float2 e2, float2 e2b, float2 e3,
                                                     float2 e3b)
 {
-    const DF2 d1 = two_diff2(e1, e1b), d2 = two_diff2(e2, e2b), d3 = two_diff2(e3, e3b);
-    const DF2 s1 = two_sum2(d1.h, d2.h), s2 = two_sum2(s1.h, d3.h);
-    const float2 sl = ad(ad(s1.l, s2.l), ad(ad(d1.l, d2.l), d3.l));
-    const DF2 a = two_prod2(fr, pi), b = two_prod2(fi, pr);
-    const DF2 c = two_diff2(a.h, b.h);
-    const float2 cl = ad(c.l, sb(a.l, b.l));
-    const float2 dh = pk(g_div.h), dl = pk(g_div.l), ph = pk(g_phi.h), pl0 = pk(g_phi.l);
-    const DF2 p = two_prod2(dh, s2.h), q = two_prod2(ph, c.h);
-    const float2 pl = ad(p.l, fm(dh, sl, ml(dl, s2.h)));
-    const float2 ql = ad(q.l, fm(ph, cl, ml(pl0, c.h)));
-    const DF2 g = two_sum2(p.h, q.h);
-    const float2 t = ad(g.l, ad(pl, ql)), h = ad(g.h, t);
-    return { { h, sb(t, sb(h, g.h)) }, ad(abs2(p.h), abs2(q.h)) };
+    const DF2 div = df_add2(df_add2(two_diff2(e1, e1b), two_diff2(e2, e2b)), two_diff2(e3, e3b));
+    const DF2 p = df_mul2(g_div, div), q = df_mul2(g_phi, df_sub2(two_prod2(fr, pi), two_prod2(fi, pr)));
+    return { df_add2(p, q), ad(abs2(p.h), abs2(q.h)) };
 }
 
 // site_phase of both sites
