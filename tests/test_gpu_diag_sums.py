@@ -1,4 +1,5 @@
-"""Precision of the whole-lattice sums of an FP32 state (GPU): the Gauss residual."""
+"""Precision of the whole-lattice sums of an FP32 state (GPU): the Gauss residual, and
+what the sums keep of the single values."""
 import numpy as np
 import pytest
 
@@ -42,3 +43,18 @@ def test_gauss_residual_of_cancelling_fields(N):
     print("\n%d^3: %.6g, relative error %.3g" % (N, exact["gauss_max"], fast["gauss_max"] / exact["gauss_max"] - 1))
     assert 0 < exact["gauss_max"] < 1e-5
     assert abs(fast["gauss_max"] - exact["gauss_max"]) <= 2.0 ** -44 * exact["gauss_max"]
+
+
+@pytest.mark.parametrize("N", [33, 44])
+def test_sums_take_every_row_by_itself(N):
+    """K = 1 in even rows and 1 + 2^-23 in odd ones: every partial sum is a multiple of
+    2^-23, so compensated sums are exact, and the FP64 total is to its own rounding."""
+    f = np.zeros((10, N, N, N))
+    f[0] = 1.0
+    f[2] = 1.0
+    f[3, :, 1::2] = np.float32(2.0 ** -11.5)
+    got = observables(N, f)["sums"][3]
+    odd = N // 2
+    ref = N * N * (N + odd * 2.0 ** -23)
+    print("\n%d^3: relative error %.3g" % (N, got / ref - 1))
+    assert abs(got - ref) <= 2.0 ** -40 * ref
