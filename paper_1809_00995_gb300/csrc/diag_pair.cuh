@@ -170,13 +170,13 @@ struct DiagPairGeo {
     static constexpr size_t smem = off_a + 2 * 4 * NE;
 };
 
-template <typename IT>
-struct DiagPair : DiagTile<float, IT> {
+template <typename IT, bool G64>
+struct DiagPair : DiagTile<float, IT, G64> {
     using G = DiagPairGeo;
-    using Base = DiagTile<float, IT>;
+    using Base = DiagTile<float, IT, G64>;
 
     // planes [z0, z1) of the 32 x 16 sites at (x0, y0)
-    __device__ __forceinline__ void column(const View<float> &v, int N, const DiagArgs &da, const SiteCoef<float> &sc,
+    __device__ __forceinline__ void column(const View<float> &v, int N, const DiagArgs &da, const typename Base::Coef &sc,
                                            int x0, int y0, int z0, int z1, unsigned char *smem)
     {
         const int lx = threadIdx.x & 31, wp = threadIdx.x >> 5;
@@ -361,10 +361,22 @@ struct DiagPair : DiagTile<float, IT> {
                 const float2 L = sb(ad(sb(KV_, G2), Eel), B);
                 const float2 rho = ad(ad(ad(K, G2), V), EB);
                 const float2 pp = fm(EB, pk(1.0f / 3.0f), fm(G2, pk(-1.0f / 3.0f), KV_));
-                const GaussTerms2 gt = gauss_terms2(sc.g_div, sc.g_phi, f0r, f0i, pr, pim, e1, e1b, e2, e2b, e3, e3m);
-                const float2 sg = ml(gt.g.h, pk(0x1p30f)), ss = ml(gt.scale, pk(0x1p30f));
-                const float2 val[13] = { K, G2, V, Eel, B, ml(K, V), ml(G2, V), ml(K, L), ml(G2, L), ml(pp, L),
-                                         ml(rho, L), ml(sg, sg), ml(ss, ss) };
+                [[maybe_unused]] GaussTerms2 gt;
+                [[maybe_unused]] GaussTerms64 ga, gb;
+                if constexpr (G64) {
+                    const DF2 a = two_prod2(f0r, pim), b = two_prod2(f0i, pr);
+                    ga = gauss_terms64(sc, { a.h.x, a.l.x }, { b.h.x, b.l.x }, e1.x, e1b.x, e2.x, e2b.x, e3.x, e3m.x);
+                    gb = gauss_terms64(sc, { a.h.y, a.l.y }, { b.h.y, b.l.y }, e1.y, e1b.y, e2.y, e2b.y, e3.y, e3m.y);
+                } else {
+                    gt = gauss_terms2(sc.g_div, sc.g_phi, f0r, f0i, pr, pim, e1, e1b, e2, e2b, e3, e3m);
+                }
+                constexpr int sums = G64 ? 11 : 13;
+                float2 val[13] = { K, G2, V, Eel, B, ml(K, V), ml(G2, V), ml(K, L), ml(G2, L), ml(pp, L), ml(rho, L) };
+                if constexpr (!G64) {
+                    const float2 sg = ml(gt.g.h, pk(0x1p30f)), ss = ml(gt.scale, pk(0x1p30f));
+                    val[11] = ml(sg, sg);
+                    val[12] = ml(ss, ss);
+                }
                 auto biggest = [&](float h, float l) {
                     if (h < 0.f) { h = -h; l = -l; }
                     if (h > this->fgmax.h || (h == this->fgmax.h && l > this->fgmax.l)) this->fgmax = { h, l };
@@ -377,14 +389,20 @@ struct DiagPair : DiagTile<float, IT> {
                 // every term of rho is >= 0, and |L|, |p| <= rho: they are finite if it is
                 if (own0) {
                     this->ic[7] += !isfinite(rho.x);
-                    biggest(gt.g.h.x, gt.g.l.x);
+                    if constexpr (G64)
+                        this->add(ga);
+                    else
+                        biggest(gt.g.h.x, gt.g.l.x);
                     this->tmax = fmaxf(this->tmax, fmaxf(fabsf(t0[0].x), fmaxf(fabsf(t0[1].x), fabsf(t0[2].x))));
                     if (own1) {
                         this->ic[7] += !isfinite(rho.y);
-                        biggest(gt.g.h.y, gt.g.l.y);
+                        if constexpr (G64)
+                            this->add(gb);
+                        else
+                            biggest(gt.g.h.y, gt.g.l.y);
                         this->tmax = fmaxf(this->tmax, fmaxf(fabsf(t0[0].y), fmaxf(fabsf(t0[1].y), fabsf(t0[2].y))));
 #pragma unroll
-                        for (int k = 0; k < 13; ++k) {
+                        for (int k = 0; k < sums; ++k) {
                             // one after the other, compensated each: their plain sum would
                             // round (and save 1.5 % of the pass, 512^3 2.86 -> 2.82 ms)
                             sum(k, val[k].x);
@@ -392,7 +410,7 @@ struct DiagPair : DiagTile<float, IT> {
                         }
                     } else {
 #pragma unroll
-                        for (int k = 0; k < 13; ++k) sum(k, val[k].x);
+                        for (int k = 0; k < sums; ++k) sum(k, val[k].x);
                     }
                 }
                 e3m = e3;

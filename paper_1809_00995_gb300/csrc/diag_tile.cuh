@@ -28,6 +28,8 @@
 // (this walk serves N that are no multiple of 4 or below 40, diag_pair.cuh the
 // others), FP64 256^3 14.9 -> 5.5 ms.
 #pragma once
+#include <cmath>
+
 #include "diag_common.cuh"
 #include "fused_common.cuh"
 #include "sincos32.cuh"
@@ -290,12 +292,23 @@ template <typename real> struct alignas(2 * sizeof(real)) D2 { real a, b; };
 // kernel took a third of the FP64 pipe.
 template <typename real> struct SiteCoef;
 template <> struct SiteCoef<float> { float inv_dx2, v_coef, eel_coef, b_coef, sigma2; DF g_div, g_phi; };
+struct SiteCoef64 : SiteCoef<float> {
+    double g_div64, g_phi64, g_div_tiny, g_phi_tiny;       // FP64, and times 2^896
+    bool tiny_ok;                                          // the latter two are finite
+};
+template <typename real, bool G64> struct PassCoef { using type = SiteCoef<real>; };
+template <> struct PassCoef<float, true> { using type = SiteCoef64; };
 struct D1 { double h; };
 template <> struct SiteCoef<double> { double inv_dx2, v_coef, eel_coef, b_coef, sigma2; D1 g_div, g_phi; };
 inline SiteCoef<float> site_coef(const DiagCoef &d, float)
 {
     return { (float)d.inv_dx2, (float)d.v_coef, (float)d.eel_coef, (float)d.b_coef, (float)d.sigma2, df_from(d.g_div),
              df_from(d.g_phi) };
+}
+inline SiteCoef64 site_coef64(const DiagCoef &d)
+{
+    const double a = d.g_div * 0x1p896, b = d.g_phi * 0x1p896;
+    return { site_coef(d, 0.f), d.g_div, d.g_phi, a, b, std::isfinite(a) && std::isfinite(b) };
 }
 inline SiteCoef<double> site_coef(const DiagCoef &d, double)
 {
@@ -310,9 +323,46 @@ struct DiagGeo {
     template <typename real> static constexpr size_t smem = 2 * (size_t)((bytes<real> + 15) / 16 * 16);
 };
 
-template <typename real, typename IT>
+// Gauss residual G and scale = |g_div div E| + |g_phi Im(conj(phi) Pi)| of FP32 fields in
+// FP64.
+struct GaussTerms64 {
+    double g, scale;
+    long long size;                      // the bits of |g|, 0 for NaN
+};
+__device__ __forceinline__ GaussTerms64 gauss_terms64(double g_div, double g_phi, double fr, double fi, double pr, double pi,
+                                                      double e1, double e1b, double e2, double e2b, double e3, double e3b)
+{
+    const double div = (e1 - e1b) + (e2 - e2b) + (e3 - e3b);
+    const double p = g_div * div, q = g_phi * (fr * pi - fi * pr), g = p + q;
+    return { g, fabs(p) + fabs(q), isnan(g) ? 0 : __double_as_longlong(fabs(g)) };
+}
+// The same of finite fields (a, b: the exact products fr pi and fi pr).  An FP64
+// instruction costs as much as 30 others here, and so does a conversion from FP32; with
+// 24 of them per site the 200^3 pass took 548 us, against 248 without.  So the bits of
+// a float are moved to where a double has them, which gives its value times 2^-896
+// (zero and subnormal ones too) in three integer instructions, and the coefficients
+// bring the factor back; |p| + |q| is the larger of |p + q| and |p - q|; and the largest
+// |G| is found in integers: 13 FP64 instructions, 372 us.
+__device__ __forceinline__ double tiny(float f)
+{
+    const int b = __float_as_int(f);
+    return __hiloint2double((b >> 3) & (int)0x8fffffff, b << 29);
+}
+__device__ __forceinline__ GaussTerms64 gauss_terms64(const SiteCoef64 &sc, DF a, DF b, float e1, float e1b, float e2,
+                                                      float e2b, float e3, float e3b)
+{
+    const double div = ((tiny(e1) - tiny(e1b)) + (tiny(e2) - tiny(e2b))) + (tiny(e3) - tiny(e3b));
+    const double q = sc.g_phi_tiny * ((tiny(a.h) - tiny(b.h)) + (tiny(a.l) - tiny(b.l)));
+    const double s = fma(sc.g_div_tiny, div, q), d = fma(sc.g_div_tiny, div, -q);
+    const long long m = 0x7fffffffffffffffLL, sa = __double_as_longlong(s) & m, da = __double_as_longlong(d) & m;
+    return { s, __longlong_as_double(max(sa, da)), sa };
+}
+// Gauss residual and its sums in FP64: of FP64 states, and of FP32 states in passes that
+// ask for it (G64).
+template <typename real, typename IT, bool G64 = sizeof(real) == 8>
 struct DiagTile {
     using G = DiagGeo;
+    using Coef = typename PassCoef<real, G64>::type;
     static constexpr int EX = G::EX, NE = G::NE;
     // sums 3..13 of ah_obs (compensated for FP32), Gauss sums and maxima, windings
     Acc<real> s[11];
@@ -323,7 +373,7 @@ struct DiagTile {
     int ic[kNumInt] = { 0, 0, 0, 0, 0, 0, 0, 0 };
 
     // one column of tiles: planes [z0, z1) of the 32 x 8 sites at (x0, y0)
-    __device__ __forceinline__ void column(const View<real> &v, int N, const DiagArgs &da, const SiteCoef<real> &sc, int x0,
+    __device__ __forceinline__ void column(const View<real> &v, int N, const DiagArgs &da, const Coef &sc, int x0,
                                            int y0, int z0, int z1, unsigned char *smem)
     {
         const int lx = threadIdx.x & 31, wy = threadIdx.x >> 5;
@@ -460,7 +510,7 @@ struct DiagTile {
         __syncthreads();                         // the next column reuses the arrays
     }
 
-    __device__ __forceinline__ void site(const SiteCoef<real> &sc, const real f0[2], const real t0[3],
+    __device__ __forceinline__ void site(const Coef &sc, const real f0[2], const real t0[3],
                                          const real sn[3], const real co[3], const D4<real> &qx, const D4<real> &qy,
                                          const real nf[2], real bsum, real pr, real pim, real e1, real e2, real e3,
                                          real e1b, real e2b, real e3b)
@@ -494,6 +544,8 @@ struct DiagTile {
             dg2 += Gs * Gs;
             dgs2 += gs * gs;
             dgmax = fmax(dgmax, fabs(Gs));
+        } else if constexpr (G64) {
+            add(gauss_terms64(sc, two_prod(f0[0], pim), two_prod(f0[1], pr), e1, e1b, e2, e2b, e3, e3b));
         } else {
             const GaussTerms gt = gauss_terms(sc.g_div, sc.g_phi, f0[0], f0[1], pr, pim, e1, e1b, e2, e2b, e3, e3b);
             DF Gs = gt.g;
@@ -506,6 +558,29 @@ struct DiagTile {
         }
     }
 
+    __device__ __forceinline__ void add(const GaussTerms64 &t)
+    {
+        dg2 += t.g * t.g;
+        dgs2 += t.scale * t.scale;
+        dgmax = __longlong_as_double(max(__double_as_longlong(dgmax), t.size));
+    }
+
+    // dg2, dgs2 and dgmax of a column again, with conversions: any fields
+    __device__ __forceinline__ void gauss_again(const View<real> &v, int N, const Coef &sc, int x0, int y0, int rows,
+                                                int z0, int z1)
+    {
+        const int x = x0 + (threadIdx.x & 31);
+        const IT NN = (IT)N * (IT)N;
+        for (int z = z0; z < z1; ++z) {
+            for (int y = y0 + (threadIdx.x >> 5); y < min(y0 + rows, N) && x < N; y += 8) {
+                const IT s = (IT)z * NN + (IT)(N * y + x), sx = x ? s - 1 : s + (N - 1), sy = y ? s - N : s + (NN - N);
+                const IT sz = z ? s - NN : s + (NN * N - NN);
+                add(gauss_terms64(sc.g_div64, sc.g_phi64, v.phr[s], v.phi[s], v.pir[s], v.pii[s], v.e1[s], v.e1[sx], v.e2[s],
+                                  v.e2[sy], v.e3[s], v.e3[sz]));
+            }
+        }
+    }
+
     __device__ __forceinline__ void flush(DiagPartial *out)
     {
         double accd[kNumSums];
@@ -515,7 +590,7 @@ struct DiagTile {
         accd[0] = accd[3] - accd[4] - accd[5] + accd[6] - accd[7];
         accd[1] = accd[3] + accd[4] + accd[5] + accd[6] + accd[7];
         accd[2] = accd[3] - accd[4] * (1.0 / 3.0) - accd[5] + (accd[6] + accd[7]) * (1.0 / 3.0);
-        if constexpr (sizeof(real) == 4) {
+        if constexpr (!G64) {
             dg2 = fg2.value() * 0x1p-60;
             dgs2 = fgs2.value() * 0x1p-60;
             dgmax = (double)fgmax.h + (double)fgmax.l;

@@ -421,32 +421,51 @@ int diag_grid_blocks(int num_sms) { return num_sms * 4; }
 
 // ------------------------------------------------------------------ whole lattice
 namespace {
+// The Gauss sums of all of a CTA's columns again, with conversions, where one of its
+// threads met a field that is not finite: a site of its own, which rho tells, or a
+// backward neighbour's E, which the moved bits make 2^128 or more; or where the
+// coefficients leave the range of gauss_terms64's factor.  (Asking at every site took
+// 27 us of the 200^3 pass.)
+template <typename T>
+__device__ __forceinline__ void gauss_of_wild_fields(T &t, const View<float> &v, int N, int tx, int ty, int items, int zc,
+                                                     int rows, const SiteCoef64 &sc)
+{
+    if (!__syncthreads_or(t.ic[7] != 0 || !(t.dgmax < sc.g_div64 * 0x1p120) || !sc.tiny_ok)) return;
+    t.dg2 = t.dgs2 = t.dgmax = 0.0;
+    for (int it = blockIdx.x; it < items; it += gridDim.x) {
+        const int bx = it % tx, by = (it / tx) % ty, z0 = it / (tx * ty) * zc;
+        t.gauss_again(v, N, sc, 32 * bx, rows * by, rows, z0, min(z0 + zc, N));
+    }
+}
+
 // Persistent CTAs over the work items (tile column, chunk of z planes), each
 // taking every gridDim.x-th one; one partial per CTA.
-template <typename real, typename IT, int MINB>
+template <typename real, typename IT, int MINB, bool G64>
 __global__ void __launch_bounds__(256, MINB)
-    k_diag_whole(View<real> v, int N, int tx, int ty, int items, int zc, SiteCoef<real> sc, DiagArgs da)
+    k_diag_whole(View<real> v, int N, int tx, int ty, int items, int zc, typename PassCoef<real, G64>::type sc, DiagArgs da)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    DiagTile<real, IT> t;
+    DiagTile<real, IT, G64> t;
     for (int it = blockIdx.x; it < items; it += gridDim.x) {
         const int bx = it % tx, by = (it / tx) % ty, z0 = it / (tx * ty) * zc;
         t.column(v, N, da, sc, 32 * bx, 8 * by, z0, min(z0 + zc, N), smem_raw);
     }
+    if constexpr (G64 && sizeof(real) == 4) gauss_of_wild_fields(t, v, N, tx, ty, items, zc, 8, sc);
     t.flush(&da.partials[blockIdx.x]);
 }
 
 // The same on 32 x 16 columns, two rows per thread (diag_pair.cuh).
-template <typename IT>
+template <typename IT, bool G64>
 __global__ void __launch_bounds__(256, 2)
-    k_diag_pair(View<float> v, int N, int tx, int ty, int items, int zc, SiteCoef<float> sc, DiagArgs da)
+    k_diag_pair(View<float> v, int N, int tx, int ty, int items, int zc, typename PassCoef<float, G64>::type sc, DiagArgs da)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    DiagPair<IT> t;
+    DiagPair<IT, G64> t;
     for (int it = blockIdx.x; it < items; it += gridDim.x) {
         const int bx = it % tx, by = (it / tx) % ty, z0 = it / (tx * ty) * zc;
         t.column(v, N, da, sc, 32 * bx, 16 * by, z0, min(z0 + zc, N), smem_raw);
     }
+    if constexpr (G64) gauss_of_wild_fields(t, v, N, tx, ty, items, zc, 16, sc);
     t.flush(&da.partials[blockIdx.x]);
 }
 
@@ -481,7 +500,7 @@ DiagGrid diag_whole_grid(const View<real> &v, int N)
     return g;
 }
 
-template <typename real, typename IT>
+template <typename real, typename IT, bool G64>
 cudaError_t launch_diag_whole_it(const View<real> &v, int N, const DiagGrid &g, const DiagArgs &da, cudaStream_t st)
 {
     constexpr size_t smem = DiagGeo::smem<real>;
@@ -489,22 +508,24 @@ cudaError_t launch_diag_whole_it(const View<real> &v, int N, const DiagGrid &g, 
     static unsigned long long configured = 0;   // per device; dynamic plus static smem may pass 48 KB
     const unsigned long long dev_bit = 1ULL << device_slot();
     if (!(configured & dev_bit)) {
-        cudaError_t e = cudaFuncSetAttribute(k_diag_whole<real, IT, minb>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(k_diag_whole<real, IT, minb, G64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem);
         if (e == cudaSuccess && sizeof(real) == 4)
-            e = cudaFuncSetAttribute(k_diag_pair<IT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            e = cudaFuncSetAttribute(k_diag_pair<IT, G64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)DiagPairGeo::smem);
         if (e != cudaSuccess) return e;
         configured |= dev_bit;
     }
-    const SiteCoef<real> sc = site_coef(da.dc, real(0));
+    typename PassCoef<real, G64>::type sc;
+    if constexpr (G64 && sizeof(real) == 4) sc = site_coef64(da.dc);
+    else sc = site_coef(da.dc, real(0));
     if constexpr (sizeof(real) == 4) {
         if (g.pair) {
-            k_diag_pair<IT><<<g.ctas, 256, DiagPairGeo::smem, st>>>(v, N, g.tx, g.ty, g.items, g.zc, sc, da);
+            k_diag_pair<IT, G64><<<g.ctas, 256, DiagPairGeo::smem, st>>>(v, N, g.tx, g.ty, g.items, g.zc, sc, da);
             return cudaGetLastError();
         }
     }
-    k_diag_whole<real, IT, minb><<<g.ctas, 256, smem, st>>>(v, N, g.tx, g.ty, g.items, g.zc, sc, da);
+    k_diag_whole<real, IT, minb, G64><<<g.ctas, 256, smem, st>>>(v, N, g.tx, g.ty, g.items, g.zc, sc, da);
     return cudaGetLastError();
 }
 }  // namespace
@@ -512,11 +533,11 @@ cudaError_t launch_diag_whole_it(const View<real> &v, int N, const DiagGrid &g, 
 int fused_diag_max_ctas() { return std::max(kDiagCtas<float>, kDiagCtas<double>) * device_sm_count(); }
 
 namespace {
-template <typename real>
+template <typename real, bool G64 = sizeof(real) == 8>
 cudaError_t launch_diag_grid(const View<real> &v, int N, const DiagGrid &g, const DiagArgs &da, cudaStream_t st)
 {
-    return (long long)N * N * N < (1LL << 31) ? launch_diag_whole_it<real, int>(v, N, g, da, st)
-                                              : launch_diag_whole_it<real, long long>(v, N, g, da, st);
+    return (long long)N * N * N < (1LL << 31) ? launch_diag_whole_it<real, int, G64>(v, N, g, da, st)
+                                              : launch_diag_whole_it<real, long long, G64>(v, N, g, da, st);
 }
 }  // namespace
 
@@ -712,7 +733,7 @@ extern "C" ah_status ah_observables_noalloc(const float *const fields[10], int32
     if (g.ctas > kNoAllocBlocks)
         return host_fail(AH_ERR_CUDA, "ah_observables_noalloc: more resident CTAs than the scratch has partials");
     cudaError_t e = cudaMemsetAsync(list.count, 0, sizeof(unsigned long long), stream);
-    if (e == cudaSuccess) e = launch_diag_grid<float>(v, N, g, da, stream);
+    if (e == cudaSuccess) e = launch_diag_grid<float, true>(v, N, g, da, stream);
     if (e == cudaSuccess) {
         k_diag_sum<<<kSumWords, kSumThreads, 0, stream>>>(partials, g.ctas, result);
         k_noalloc_fixup<float><<<nblocks, 128, 0, stream>>>(v, N, list, result);
