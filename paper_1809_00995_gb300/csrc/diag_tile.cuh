@@ -65,6 +65,19 @@ __device__ __forceinline__ float site_phase(float r, float i)
     a = i < 0.f ? -a : a;
     return hi > 1e-30f && x + y < 1e30f ? a : __int_as_float(0x7fc00000);
 }
+// FP64 phi past the range above: its phase is that of phi over a power of two
+static __device__ __noinline__ float site_phase_scaled(double r, double i)
+{
+    const double m = fmax(fabs(r), fabs(i));
+    if (!(m > 0.0 && m <= 0x1.fffffffffffffp+1023)) return __int_as_float(0x7fc00000);
+    const int e = ilogb(m);
+    return site_phase((float)scalbn(r, -e), (float)scalbn(i, -e));
+}
+__device__ __forceinline__ float site_phase(double r, double i)
+{
+    const float a = site_phase((float)r, (float)i);
+    return a == a ? a : site_phase_scaled(r, i);
+}
 
 // n of a link whose bracket is a - 2 pi n, and whether the bracket is too near
 // the cut: adding 1.5 x 2^23 rounds to the nearest integer, which the low bits then
@@ -421,8 +434,8 @@ struct DiagTile {
         real e3m = v.e3[wrapz(z0 - 1) + (IT)roff];
         load_fields(z0);
         load_momenta(z0);
-        a0 = site_phase((float)nf[0], (float)nf[1]);
-        ra = fwd ? site_phase((float)rf[0], (float)rf[1]) : 0.f;
+        a0 = site_phase(nf[0], nf[1]);
+        ra = fwd ? site_phase(rf[0], rf[1]) : 0.f;
         unsigned wm = 0;                         // own turns and N of plane z - 1
         for (int z = z0; z <= z1; ++z) {
             const int b = z & 1;
@@ -451,7 +464,7 @@ struct DiagTile {
             const float ax = atf(b)[e + 1], ay = atf(b)[e + EX];
             const real e1x = at2(b)[e - 1].a, e2y = at2(b)[e - EX].b;
             if (z + 1 < z1) load_momenta(z + 1);
-            const float an = z < z1 ? site_phase((float)nf[0], (float)nf[1]) : 0.f;
+            const float an = z < z1 ? site_phase(nf[0], nf[1]) : 0.f;
             int n[3];
             int nc;
             {
@@ -461,7 +474,7 @@ struct DiagTile {
             }
             if (fwd) {
                 // the row above: n_1, n_3; the column to the right: n_2, n_3
-                const float rn = z < z1 ? site_phase((float)rf[0], (float)rf[1]) : 0.f;
+                const float rn = z < z1 ? site_phase(rf[0], rf[1]) : 0.f;
                 const float aj = above ? atf(b)[he + 1] : (lx < 8 ? atf(b)[he + EX] : 0.f);
                 const float bn[3] = { aj, aj, rn };
                 int rk[3];
