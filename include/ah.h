@@ -64,7 +64,9 @@ enum { AH_KERNEL_AUTO = 0, AH_KERNEL_PLAIN = 1, AH_KERNEL_FUSED = 2 };
 /* Configuration flags.
  *  EXACT_DIAG: evaluate every diagnostic per site in FP64 with arctangent
  *  windings (slow).  By default per-site energies are evaluated in the state
- *  precision (accumulated in FP64), the Gauss residual in FP64, and windings as
+ *  precision (FP32: compensated FP32 sums per thread, FP64 across threads), the
+ *  Gauss residual in FP64 (of an FP32 state in double-float arithmetic, its
+ *  squares in compensated FP32 sums per thread), and windings as
  *  integer turns that equal the FP64 arctangent formula, with the plaquettes
  *  near a branch cut re-evaluated in FP64. */
 enum { AH_FLAG_EXACT_DIAG = 1, AH_FLAG_AUTOTUNE = 2, AH_FLAG_WRAP_THETA = 4, AH_FLAG_CORE_GROWTH = 8,
@@ -231,7 +233,10 @@ ah_status ah_observables_finish(ah_sim *sim, ah_obs *out);
 
 /* Copy the state of the window [x0, x0+nx) x ... (mod N) to host memory `out`
  * as FP64: 10 components, each nz*ny*nx with x fastest (10*nx*ny*nz doubles).
- * Waits for the simulation's stream. */
+ * Waits for the simulation's stream.  The window goes through a device buffer of
+ * its size; the simulation keeps one of up to 64 MB (the largest window so far,
+ * here and in ah_set_fields) until ah_destroy, which ah_info.state_bytes does not
+ * count. */
 ah_status ah_get_fields(ah_sim *sim, int32_t x0, int32_t y0, int32_t z0,
                         int32_t nx, int32_t ny, int32_t nz, double *out);
 
@@ -310,7 +315,10 @@ ah_status ah_autotune(ah_sim *sim, int32_t trial_steps, int32_t *chosen);
  * (the rounds of such a batch then run without a CUDA graph).  Its results
  * agree with one step per launch to FP32 rounding.
  * The other lattices take one step per launch.  (Small lattices gain nothing
- * from pairs: the two-step tile writes 30 x 6 of its 32 x 8 sites.) */
+ * from pairs: the two-step tile writes 30 x 6 of its 32 x 8 sites.  Nor do large
+ * ones whose side is a multiple of 4, whose single step is the faster kernel;
+ * for one lattice in a batch, single steps / pairs, ms per step: 512^3 1.92 / 2.14,
+ * 1024^3 15.9 / 16.7, but 1022^3 19.1 / 17.0.) */
 enum { AH_BATCH_AUTOTUNE = 1, AH_BATCH_NO_GRAPH = 2, AH_BATCH_TWO_STEP = 4 };
 
 typedef struct ah_batch_stats {
@@ -434,9 +442,9 @@ typedef struct ah_sums {
  *           written by the call.
  *  stream   cudaStream_t (as void*) the work is enqueued on; the call returns
  *           without waiting, so read d_sums after synchronising that stream.
- * The per-site values and the sums are the same as those of ah_observables
- * (fast path: FP32 energies, FP64 sums and Gauss residual, windings equal to the
- * FP64 arctangent formula).  Scratch memory -- per-block partial sums and a list
+ * The per-site energies and their sums are those of ah_observables (FP32,
+ * compensated FP32 sums per thread, FP64 across threads), the Gauss residual and
+ * its sums are FP64, windings equal the FP64 arctangent formula.  Scratch memory -- per-block partial sums and a list
  * of at most 2^18 plaquettes near a branch cut -- lives in one static device
  * array of 2.31 MB that every GPU which loads the library holds until exit; if
  * a snapshot has more listed plaquettes than that, all windings of the call are

@@ -7,7 +7,7 @@
 // is one thread's.  Per plane and site: the three forward products U_d phi^{x+d}
 // (the gradient energy), the three plaquette phases from the link phases
 // (1 - cos Xi by its own series, without cancellation or division), and the
-// Gauss residual (double-float for FP32 states).
+// Gauss residual (double-float for FP32 states, or FP64: G64).
 //
 // Windings without arctangents per edge.  With alpha = arg phi of each site, the
 // bracket of Eq. 9 on link e from a to b is [alpha_b - alpha_a + theta_e] =
@@ -16,9 +16,9 @@
 //   W = (sum of the four brackets - [Xi]) / 2 pi = N - (n_1 + n_2 - n_3 - n_4),
 // N the nearest integer of Xi / 2 pi: one arctangent per site and small integers.
 // alpha is good to 1e-6 in FP32; where a bracket or [Xi] comes within 2^-15 of
-// +-pi (kCutMargin), or phi is too small or too large for alpha, the plaquette goes
-// to the list that the FP64 path decides, so the counts are those of the FP64
-// formula on the same state.  A site needs n_2, n_3 of x + 1 and n_1, n_3 of x + y
+// +-pi (kCutMargin), phi is too small or too large for alpha, or a phase makes
+// thousands of turns (kMaxTurns), the plaquette goes to the list that the FP64 path
+// decides, so the counts are those of the FP64 formula on the same state.  A site needs n_2, n_3 of x + 1 and n_1, n_3 of x + y
 // (one packed word each) and its own n_1, n_2 of the next plane, so the windings
 // of plane z - 1 are summed while plane z is worked on, and a plane costs one
 // barrier (two copies of the shared arrays).
@@ -26,7 +26,7 @@
 // FP32 is bound by instruction issue, FP64 by its pipe.  Against a walk with the
 // step's link exponentials and chained edge products: FP32 512^3 5.48 -> 3.95 ms
 // (this walk serves N that are no multiple of 4 or below 40, diag_pair.cuh the
-// others), FP64 256^3 14.9 -> 5.5 ms.
+// others; 381^3 1.60 ms), FP64 256^3 14.9 -> 5.7 ms.
 #pragma once
 #include <cmath>
 

@@ -12,7 +12,7 @@
 // nor a window of 40 columns wrap twice: N a multiple of 4, and at least 40.
 //
 // What it measured (512^3, ms per step): 1.69 = 6.3 TB/s, 0.93 of 6.8 TB/s, against
-// 2.06 of the one-site walk; 256^3 0.232 against 0.265; 1024^3 13.8 against 16.4.
+// 2.06 of the one-site walk; 256^3 0.231 against 0.275; 1024^3 13.8 against 16.4.
 // One plane ahead instead of two 1.98 (the copies' latency shows); rows copied whole
 // by cp.async.bulk 2.52 (170 copies of 128 or 160 bytes per plane and CTA take 22
 // cycles each); one barrier per plane, with the curls of plane z - 1 after the barrier
