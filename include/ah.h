@@ -315,10 +315,11 @@ ah_status ah_autotune(ah_sim *sim, int32_t trial_steps, int32_t *chosen);
  * (the rounds of such a batch then run without a CUDA graph).  Its results
  * agree with one step per launch to FP32 rounding.
  * The other lattices take one step per launch.  (Small lattices gain nothing
- * from pairs: the two-step tile writes 30 x 6 of its 32 x 8 sites.  Nor do large
- * ones whose side is a multiple of 4, whose single step is the faster kernel;
- * for one lattice in a batch, single steps / pairs, ms per step: 512^3 1.92 / 2.14,
- * 1024^3 15.9 / 16.7, but 1022^3 19.1 / 17.0.) */
+ * from pairs: the two-step tile writes 30 x 6 of its 32 x 8 sites.  Large ones
+ * gain where the side is no multiple of 4; otherwise the single step is as fast or
+ * faster.  One lattice in a batch, ms per step of single steps / pairs (in the form
+ * for weak gauge fields): 512^3 1.84 / 2.07 (1.94), 1024^3 14.8 / 15.5 (14.7), 1022^3
+ * 17.5 / 15.5 (14.5).) */
 enum { AH_BATCH_AUTOTUNE = 1, AH_BATCH_NO_GRAPH = 2, AH_BATCH_TWO_STEP = 4 };
 
 typedef struct ah_batch_stats {

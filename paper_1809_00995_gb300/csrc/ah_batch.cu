@@ -47,10 +47,10 @@ constexpr int kZChunk2 = 256;      // planes per two-step work item (each also r
 // smaller ones one step per launch: the two-step tile writes 30 x 6 of its
 // 32 x 8 sites, so small lattices pay more in partial tiles and halo
 // recomputation than they save in DRAM traffic.  From here on pairs win where
-// rows cannot be copied in 16 bytes (one lattice in a batch, single steps / pairs,
-// ms per step with two diagnostics passes in 20 or 40 steps: 1022^3 19.1 / 17.0);
-// where they can, feed_tile.cuh's single step has overtaken them (512^3 1.92 / 2.14,
-// 1024^3 15.9 / 16.7), and pairs are what a caller who sets the flag asks for.
+// rows cannot be copied in 16 bytes (one lattice in a batch, ms per step of single
+// steps / pairs / pairs in weak gauge fields: 1022^3 17.5 / 15.5 / 14.5); where they
+// can, feed_tile.cuh's single step is ahead at 512^3 (1.84 / 2.07 / 1.94) and level at
+// 1024^3 (14.8 / 15.5 / 14.7), and pairs are what a caller who sets the flag asks for.
 constexpr int kPairMinN = 512;
 // Paired lattices of at least this side fill the GPU with their own two-step
 // grid (512^3: 3096 CTAs): they run the single-lattice two-step kernel, whose

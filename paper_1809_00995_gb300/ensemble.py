@@ -86,7 +86,7 @@ def case_configs(ah, name, N, seeds, diag_every, seed0=1):
 def scaling_ensemble(N=512, seeds=5, cases=tuple(CASES), diag_every=10, window=0.5, two_step=True):
     """Run every case for `seeds` seeds (one batched job per case; with two_step,
     AH_BATCH_TWO_STEP: lattices of side >= 512 two leapfrog steps per launch, which
-    takes 2.14 ms per step at 512^3 against 1.92 one step per launch) and
+    takes 2.07 ms per step at 512^3 against 1.84 one step per launch) and
     return the per-run and per-case scaling quantities."""
     import paper_1809_00995_gb300 as ah
     out = {"N": N, "seeds": seeds, "diag_every": diag_every, "window": window, "two_step": two_step, "cases": {}}
