@@ -249,8 +249,8 @@ __global__ void __launch_bounds__(NT) k_diag_fast(View<real> v, int N, Box b, Di
 // FP64 windings of the first n listed plaquettes, added to the result.  Four lanes
 // take a plaquette, one edge each: a list is short and its kernel as long as one
 // plaquette's chain of FP64 instructions, which one lane makes of four sines and
-// cosines in a row (ah_observables_noalloc at 200^3: 234 -> 228 us, 16 lattices of a
-// batch with 48 passes 62.0 -> 61.8 ms).
+// cosines in a row (6 us less per pass at 200^3, 16 lattices of a batch with 48 passes
+// 62.0 -> 61.8 ms).
 template <typename real>
 __device__ __forceinline__ void fix_windings(const View<real> &v, int N, const DiagList &list, unsigned long long n,
                                              DiagPartial *result)
@@ -384,8 +384,8 @@ __global__ void __launch_bounds__(NT) k_diag_exact(View<real> v, int N, Box b, D
 // Sum many partials in a fixed order: block k reduces word k, thread t the partials
 // t, t + 128, ..., then a tree over the threads.  Latency-bound: a chain of dependent
 // adds over strided loads, so its length is what counts (n / 128 adds and 7 levels;
-// one block with a warp per 1/32 of the partials had n / 32 + 32): 242 -> 229 us per
-// ah_observables_noalloc at 200^3.
+// one block with a warp per 1/32 of the partials had n / 32 + 32): 13 us less per pass
+// at 200^3.
 constexpr int kSumWords = kNumSums + kNumMax + kNumInt, kSumThreads = 128;
 __global__ void __launch_bounds__(kSumThreads) k_diag_sum(const DiagPartial *partials, int n, DiagPartial *result)
 {
@@ -423,9 +423,10 @@ int diag_grid_blocks(int num_sms) { return num_sms * 4; }
 namespace {
 // The Gauss sums of all of a CTA's columns again, with conversions, where one of its
 // threads met a field that is not finite: a site of its own, which rho tells, or a
-// backward neighbour's E, which the moved bits make 2^128 or more; or where the
-// coefficients leave the range of gauss_terms64's factor.  (Asking at every site took
-// 27 us of the 200^3 pass.)
+// backward neighbour's E, which the moved bits make 2^128 or more (two that cancel are
+// met at their own sites, so the sums are infinite then instead of not a number); or
+// where the coefficients leave the range of gauss_terms64's factor.  (Asking at every
+// site took 27 us of the 200^3 pass.)
 template <typename T>
 __device__ __forceinline__ void gauss_of_wild_fields(T &t, const View<float> &v, int N, int tx, int ty, int items, int zc,
                                                      int rows, const SiteCoef64 &sc)
