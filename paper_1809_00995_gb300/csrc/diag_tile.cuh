@@ -350,13 +350,12 @@ __device__ __forceinline__ GaussTerms64 gauss_terms64(double g_div, double g_phi
     return { g, fabs(p) + fabs(q), isnan(g) ? 0 : __double_as_longlong(fabs(g)) };
 }
 // The same of finite fields (a, b: the products fr pi and fi pr, exact from 2^-100 on).
-// An FP64
-// instruction costs as much as 30 others here, and so does a conversion from FP32; with
-// 24 of them per site the 200^3 pass took 548 us, against 248 without.  So the bits of
-// a float are moved to where a double has them, which gives its value times 2^-896
-// (zero and subnormal ones too) in three integer instructions, and the coefficients
-// bring the factor back; |p| + |q| is the larger of |p + q| and |p - q|; and the largest
-// |G| is found in integers: 13 FP64 instructions, 372 us.
+// An FP64 instruction costs as much as 30 others here, and so does a conversion from
+// FP32; with 24 of them per site the 200^3 pass took 548 us, against 248 without.  So
+// the bits of a float are moved to where a double has them, which gives its value
+// times 2^-896 (zero and subnormal ones too) in three integer instructions, and the
+// coefficients bring the factor back; |p| + |q| is the larger of |p + q| and |p - q|; and
+// the largest |G| is found in integers: 13 FP64 instructions, 372 us.
 __device__ __forceinline__ double tiny(float f)
 {
     const int b = __float_as_int(f);
